@@ -372,7 +372,9 @@ lift_status lift_dot_ex_v(int variant, lift_dtype t, const void* x, const float*
 
 /* ------------------------------------------------------------------------
  * Variant policy.
- *   LIFT_POLICY_FIXED: the per-op default variant (or lift_set_variant's).
+ *   LIFT_POLICY_FIXED: the per-op default variant, chosen among a few by
+ *                      the call's shape and alignment where that matters
+ *                      (or lift_set_variant's); no file, no timing.
  *   LIFT_POLICY_TABLE: a tuned table (path: a text file written by the
  *                      autotuner; nearest shape in log2 size).
  *   LIFT_POLICY_MLP:   the cost model (path: weights file written by the

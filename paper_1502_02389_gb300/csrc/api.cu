@@ -153,6 +153,8 @@ void register_blackscholes(std::vector<Variant>& bs);  // blackscholes.cu
 void register_compensated(std::vector<Variant>& asum, std::vector<Variant>& dot);  // compensated.cu
 void register_reduce_derived(std::vector<Variant>& asum, std::vector<Variant>& dot);  // reduce_derived.cu
 void gemv_split_shape(int k, const Args& a, int64_t* L, int64_t* S);
+void register_gemv_rows(std::vector<Variant>& gemv);   // gemv_rows.cu (several rows at a time)
+void gemv_split_rows_shape(const char* name, const Args& a, int64_t* L, int64_t* S);
 lift_status gemv_t_empty_rows(int64_t N, float beta, float* y, cudaStream_t s);
 
 static std::vector<Variant> g_ops[LIFT_NUM_OPS];
@@ -168,6 +170,7 @@ static void build_registry() {
   register_gemv_split(g_ops[LIFT_OP_GEMV]);
   register_gemv_tmap(g_ops[LIFT_OP_GEMV]);
   register_gemv_pertile(g_ops[LIFT_OP_GEMV]);
+  register_gemv_rows(g_ops[LIFT_OP_GEMV]);
   register_mixed(g_ops);
   register_axpy(g_ops[LIFT_OP_AXPY]);
   register_gemv_t(g_ops[LIFT_OP_GEMV_T]);
@@ -261,8 +264,9 @@ static std::mutex g_policy_mu;
 
 // Defaults of the FIXED policy: per op, a variant that is the autotuner's
 // best or within a few per cent of it at the benchmark configurations of that
-// op on the GB300 (the learned and table policies adapt to other shapes).
-// Variant names; looked up at first use.
+// op on the GB300.  For the ops whose best form depends on the shape or the
+// alignment, fixed_pick below chooses among a few more.  Variant names;
+// looked up at first use.
 static const char* kDefaultName[LIFT_NUM_OPS] = {
     "asum_t4096_v4_ldg_p2", "dot_t4096_v4_ldg_p2", "scal_t2048_v4_ldg_pertile",
     "gemv_tma_w4_c1024_s3", "asum_bf16_t256_u4", "dot_bf16_t256_u4", "asum_fp8_t256_u8_c",
@@ -326,6 +330,56 @@ static bool eligible(int op, const Variant& v, const Args& a) {
   // tensor copies: whole 256-float runs per row, 16-byte row strides
   if (op == LIFT_OP_GEMV && v.info.tree == 3) ok = ok && a.N % 256 == 0 && a.lda % 4 == 0;
   return ok;
+}
+
+// The FIXED policy.  gemv: by the row length, the number of rows and whether
+// rows can be read in 16-byte vectors.  Times in us on a GB300, graph of
+// back-to-back calls on cold data:
+//  * rows in 16-byte granules, N >= 2048: the bulk-copy ring gives each CTA
+//    whole rows, which needs rows enough for every SM: it leads from about
+//    2000 rows on (2400 x 32768: 49 against 53 for the split rows); below
+//    that the rows are split over CTAs (600 x 131072: 48 against 80;
+//    64 x 32768: 4.3 against 16).  A few rows of one ring's length stay with
+//    the ring: no second pass (64 x 4096: 3.0 against 3.5).
+//  * N < 2048: a warp per row, as the ring's stages would be mostly empty
+//    (20000 x 1024: 16.1 against 17; 80000 x 64: 16.9 against 44);
+//    8-float loads from 256 columns on, where one row fills a warp's load.
+//  * rows in 4-byte granules (N, lda or a pointer off 16 bytes): the forms
+//    that fold several rows at a time.  From 1024 columns on a CTA per row
+//    group (8193 x 5000: 29 against 62 for a warp per row), R = 4 rows where
+//    x is long enough to be read from L2 each time (N >= 65536) or the rows
+//    are short and many; below, two rows per warp (80000 x 65: 13.3 against
+//    17.2 one at a time).
+static int fixed_gemv(const Args& a) {
+  enum { kRing, kRing4, kSplit4, kWarp8, kWarp4, kSplit1R4, kSplit1R2, kSplit1Short, kWarp1, kCount };
+  static const char* const names[kCount] = {
+      "gemv_tma_w2_c2048_s3",     "gemv_tma_w4_c1024_s3",     "gemv_split_t128_v4_r2_u4",
+      "gemv_w4_v8_u2_pertile",    "gemv_w8_v4_u8",            "gemv_split_t256_v1_r4_u8",
+      "gemv_split_t256_v1_r2_u8", "gemv_split_t128_v1_r4_u8", "gemv_w4_v1_r2_u8"};
+  static const std::vector<int> id = [] {
+    std::vector<int> v;
+    for (const char* n : names) v.push_back(find_variant(LIFT_OP_GEMV, n));
+    return v;
+  }();
+  const auto& L = registry(LIFT_OP_GEMV);
+  auto ok = [&](int k) { return eligible(LIFT_OP_GEMV, L[id[k]], a); };
+  const int64_t M = a.M, N = a.N;
+  if (ok(kWarp4)) {                     // 16-byte granules
+    if (N < 256) return id[kWarp4];
+    if (N < 2048) return id[ok(kWarp8) ? kWarp8 : kWarp4];
+    const bool few = N < 4096 ? M >= 1000 && M < 2000 : N < 8192 ? M >= 500 && M < 2000 : M < 2000;
+    if (few) return id[kSplit4];
+    const int ring = N < 4096 && M >= 2000 ? kRing4 : kRing;
+    return id[ok(ring) ? ring : kSplit4];
+  }
+  if (N < 1024) return id[kWarp1];
+  if (N >= 65536) return id[kSplit1R4];
+  return id[N < 4096 && M >= 4000 ? kSplit1Short : kSplit1R2];
+}
+
+static int fixed_pick(int op, const Args& a) {
+  if (op == LIFT_OP_GEMV) return fixed_gemv(a);
+  return find_variant(op, kDefaultName[op]);
 }
 
 // The learned ranking: (predicted log-time, variant) of every variant that
@@ -577,7 +631,8 @@ static int tune_candidates(int op, const Args& a0, const std::vector<int>& cand,
   return best;
 }
 
-static int pick_variant(int op, const Args& a, cudaStream_t s = nullptr, bool may_tune = false) {
+static int pick_variant(int op, const Args& a, cudaStream_t s = nullptr, bool may_tune = false,
+                        bool by_shape = true) {
   std::unique_lock<std::mutex> lk(g_policy_mu);
   if (g_override[op] >= 0) return g_override[op];
   int v = -1;
@@ -614,7 +669,7 @@ static int pick_variant(int op, const Args& a, cudaStream_t s = nullptr, bool ma
         };
         for (size_t i = 0; i < r.size() && (int)i < kTuneTopK; ++i) add(r[i].second);
         const auto& L = registry(op);
-        const int fixed = find_variant(op, kDefaultName[op]);
+        const int fixed = fixed_pick(op, a);
         if (fixed >= 0 && eligible(op, L[fixed], a)) add(fixed);
         const int known = (op + 1 < g_mlp.ops ? g_mlp.offsets[op + 1] : g_mlp.V) - g_mlp.offsets[op];
         for (int i = known; i < (int)L.size(); ++i)      // newer than the model
@@ -638,8 +693,20 @@ static int pick_variant(int op, const Args& a, cudaStream_t s = nullptr, bool ma
     }
   }
   if (g_policy == LIFT_POLICY_TABLE) v = table_pick(op, a);
-  if (v < 0) v = find_variant(op, kDefaultName[op]);
+  if (v < 0) v = by_shape ? fixed_pick(op, a) : find_variant(op, kDefaultName[op]);
   return v;
+}
+
+// The pick whose tile and vector width a batched op takes: the policy's,
+// except that FIXED means each op's one default (the shape rules choose
+// between launches, which a batch's work items do not have).
+int batch_pick(int op, int64_t n, int64_t M, int64_t N) {
+  Args a;
+  a.n = n;
+  a.M = M;
+  a.N = N;
+  a.lda = N;
+  return pick_variant(op, a, nullptr, false, false);
 }
 
 // Resolve the variant to run: explicit id or policy pick, then the guarded
@@ -1134,11 +1201,13 @@ lift_status lift_gemv_segments(int variant, int64_t M, int64_t N, int64_t* seg_l
     *segments = 1;
     return LIFT_OK;
   }
-  int first = variant;
-  while (first > 0 && strncmp(L[first - 1].info.name, "gemv_split_", 11) == 0) --first;
   Args a;
   a.M = M;
   a.N = N;
+  gemv_split_rows_shape(L[variant].info.name, a, seg_len, segments);
+  if (*segments > 0) return LIFT_OK;
+  int first = variant;
+  while (first > 0 && strncmp(L[first - 1].info.name, "gemv_split_", 11) == 0) --first;
   gemv_split_shape(variant - first, a, seg_len, segments);
   return LIFT_OK;
 }

@@ -19,7 +19,7 @@
 // queue, and lets the hardware deal the CTAs to the SMs as earlier ones
 // retire; the items, their order and the combine are the same.
 //
-// Per op, the policy's variant choice (lift_pick: FIXED, TABLE or MLP) is
+// Per op, the policy's variant choice (batch_pick: FIXED, TABLE or MLP) is
 // mapped to a processing mode: vector ops take the (tile, vector width) of
 // the chosen variant when the batch kernel has that mode, gemv takes its
 // vector width.  A pointer that is not aligned for the mode's vector width
@@ -406,7 +406,7 @@ lift_status lift_batch_create(const lift_op_desc* descs, int64_t count, lift_bat
     o.A = d.A;
     o.out = d.out;
     int v = d.variant;
-    if (v < 0) lift_pick(d.op, d.n, d.M, d.N, &v);
+    if (v < 0) v = batch_pick(d.op, d.n, d.M, d.N);
     b->variant[i] = v;
     const lift_variant_info& info = registry(d.op)[v].info;
     o.first_item = (int64_t)items.size();

@@ -84,6 +84,7 @@ struct Variant {
 };
 
 std::vector<Variant>& registry(int op);
+int batch_pick(int op, int64_t n, int64_t M, int64_t N);   // the pick of a batched op
 
 void register_reduce_f32(std::vector<Variant>& asum, std::vector<Variant>& dot);
 void register_scal(std::vector<Variant>& scal);

@@ -1,0 +1,59 @@
+"""The FIXED policy's choices by shape and alignment: the default entry points
+on both sides of every threshold, with matrices whose rows, pointers and
+vectors are and are not whole 16-byte granules, against the FP64 oracle
+within the parity bound."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from oracle import blas
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def L():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1502_02389_gb300 import build, lift
+    build.build()
+    torch.cuda.set_device(0)
+    lift.lift_init(0)
+    yield lift
+    torch.cuda.synchronize()
+    assert lift.lift_read_status() == 0
+
+
+def at(a, off):
+    """A device copy of the fp32 array a, `off` elements past a 256-byte
+    boundary, NaN around it: (buffer, address)."""
+    b = torch.full((a.size + 128,), float("nan"), device="cuda")
+    b[64 + off:64 + off + a.size] = torch.from_numpy(np.ascontiguousarray(a).reshape(-1)).cuda()
+    return b, b.data_ptr() + 4 * (64 + off)
+
+
+# (M, N) around the rules' thresholds, ragged and whole; (pad, offsets of A, x, y)
+FORMS = [(0, 0, 0, 0), (0, 1, 2, 3), (1, 0, 0, 0), (4, 0, 0, 1), (8, 0, 0, 0)]
+GEMV = [(1, 1), (3, 0), (7, 255), (7, 256), (40, 1023), (9, 1024), (5, 2047), (999, 2048),
+        (1000, 2048), (2000, 2050), (499, 4096), (500, 4097), (3, 8192), (2000, 8192), (4000, 1025),
+        (4001, 3001), (2, 65535), (3, 65536), (5, 70003)]
+
+
+@pytest.mark.parametrize("M,N", GEMV)
+def test_gemv(L, M, N):
+    rng = np.random.default_rng(M * 131 + N)
+    A = rng.uniform(-1, 1, (M, N)).astype(np.float32)
+    x, y = rng.uniform(-1, 1, N).astype(np.float32), rng.uniform(-1, 1, M).astype(np.float32)
+    for pad, oa, ox, oy in FORMS:
+        Ap = np.full((M, N + pad), np.nan, np.float32)
+        Ap[:, :N] = A
+        bufs = [at(Ap, oa), at(x, ox)]
+        for beta in (0.5, 0.0):
+            out, py = at(y, oy)
+            L.lift_gemv(M, N, 1.25, bufs[0][1], N + pad, bufs[1][1], beta, py)
+            got = out[64 + oy:64 + oy + M].cpu().numpy().astype(np.float64)
+            ref = blas.gemv(A.astype(np.float64), x.astype(np.float64), y.astype(np.float64), 1.25, beta)
+            tol = blas.tolerance(max(N, 2), 1.0) * blas.gemv_row_terms(A, x, y, 1.25, beta)
+            assert np.all(np.abs(got - ref) <= tol), (pad, oa, ox, oy, beta)
+            assert torch.isnan(out[:64 + oy]).all() and torch.isnan(out[64 + oy + M:]).all()
