@@ -147,6 +147,8 @@ void register_reduce_f32(std::vector<Variant>& asum, std::vector<Variant>& dot,
 void register_axpy(std::vector<Variant>& axpy);       // scal_gemv.cu
 void register_gemv_t(std::vector<Variant>& gemv_t);   // gemv_t.cu
 void gemv_t_shape(int id, const Args& a, int64_t* B, int64_t* RB);
+void register_gemv_t_cols(std::vector<Variant>& gemv_t);  // gemv_t_cols.cu
+void gemv_t_cols_shape(const char* name, const Args& a, int64_t* B, int64_t* RB);
 void register_gemv_split(std::vector<Variant>& gemv);  // gemv_split.cu
 void register_gemv_pertile(std::vector<Variant>& gemv);  // scal_gemv.cu (one CTA per row group)
 void register_blackscholes(std::vector<Variant>& bs);  // blackscholes.cu
@@ -174,6 +176,7 @@ static void build_registry() {
   register_mixed(g_ops);
   register_axpy(g_ops[LIFT_OP_AXPY]);
   register_gemv_t(g_ops[LIFT_OP_GEMV_T]);
+  register_gemv_t_cols(g_ops[LIFT_OP_GEMV_T]);
   register_blackscholes(g_ops[LIFT_OP_BLACKSCHOLES]);
   register_compensated(g_ops[LIFT_OP_ASUM_COMP], g_ops[LIFT_OP_DOT_COMP]);
 }
@@ -377,8 +380,41 @@ static int fixed_gemv(const Args& a) {
   return id[N < 4096 && M >= 4000 ? kSplit1Short : kSplit1R2];
 }
 
+// gemv-T, the same way (us):
+//  * 4-byte granules: strided columns per thread (4097 x 3001: 13.2 against
+//    31.5 for the one-pass 4-byte form; 20000 x 513: 12.2 against 85).
+//  * 16-byte granules, and more columns than 8 times the rows: the same
+//    family, which has no second pass once the columns fill a wave
+//    (32 x 1000000: 23.5 against 144 for the staged form), in 16-byte loads
+//    from 16384 columns on (1200 x 32768: 26.1 against 29).  Also for small
+//    matrices (M <= 128, or N <= 512 with fewer than 10000 rows), where a
+//    ring has no time to fill: 64 x 2048: 3.1 against 4.0.
+//  * otherwise the staged form: 32 consumer threads (128 columns) per CTA for
+//    up to 256 columns (80000 x 64: 10.4 against 13.6), 64 below 4096
+//    columns (5000 x 2048: 10.9 against 11.2), 128 from there on (gemv and
+//    gemv-T of 8192 x 8192 in turn: 80.6 against 82.2).
+static int fixed_gemv_t(const Args& a) {
+  enum { kCols1, kCols4, kStaged, kStagedMid, kStagedNarrow, kCount };
+  static const char* const names[kCount] = {"gemv_t_t128_v1_q2_u8_p2", "gemv_t_t128_v4_q1_u8_p2",
+                                            "gemv_t_t128_v4_r16_s3", "gemv_t_t64_v4_r32_s3",
+                                            "gemv_t_t32_v4_r32_s3"};
+  static const std::vector<int> id = [] {
+    std::vector<int> v;
+    for (const char* n : names) v.push_back(find_variant(LIFT_OP_GEMV_T, n));
+    return v;
+  }();
+  const auto& L = registry(LIFT_OP_GEMV_T);
+  auto ok = [&](int k) { return eligible(LIFT_OP_GEMV_T, L[id[k]], a); };
+  const int64_t M = a.M, N = a.N;
+  const bool wide = N / 8 >= M;
+  if (wide && N >= 16384 && ok(kCols4)) return id[kCols4];
+  if (wide || M <= 128 || (N <= 512 && M < 10000) || !ok(kStaged)) return id[kCols1];
+  return id[N <= 256 ? kStagedNarrow : N < 4096 ? kStagedMid : kStaged];
+}
+
 static int fixed_pick(int op, const Args& a) {
   if (op == LIFT_OP_GEMV) return fixed_gemv(a);
+  if (op == LIFT_OP_GEMV_T) return fixed_gemv_t(a);
   return find_variant(op, kDefaultName[op]);
 }
 
@@ -1161,6 +1197,8 @@ lift_status lift_gemv_t_blocks(int variant, int64_t M, int64_t N, int64_t* rows_
   Args a;
   a.M = M;
   a.N = N;
+  gemv_t_cols_shape(registry(LIFT_OP_GEMV_T)[variant].info.name, a, rows_per_block, blocks);
+  if (*blocks > 0) return LIFT_OK;
   gemv_t_shape(variant, a, rows_per_block, blocks);
   return LIFT_OK;
 }

@@ -57,3 +57,29 @@ def test_gemv(L, M, N):
             tol = blas.tolerance(max(N, 2), 1.0) * blas.gemv_row_terms(A, x, y, 1.25, beta)
             assert np.all(np.abs(got - ref) <= tol), (pad, oa, ox, oy, beta)
             assert torch.isnan(out[:64 + oy]).all() and torch.isnan(out[64 + oy + M:]).all()
+
+
+GEMV_T = [(1, 1), (0, 5), (5, 3), (33, 256), (128, 300), (129, 512), (129, 513), (9999, 100),
+          (10000, 256), (10001, 257), (130, 1040), (130, 1044), (2048, 16384), (2049, 16380), (3, 65536),
+          (70, 40001), (300, 600)]
+
+
+@pytest.mark.parametrize("M,N", GEMV_T)
+def test_gemv_t(L, M, N):
+    rng = np.random.default_rng(M * 137 + N)
+    A = rng.uniform(-1, 1, (M, N)).astype(np.float32)
+    x, y = rng.uniform(-1, 1, M).astype(np.float32), rng.uniform(-1, 1, N).astype(np.float32)
+    A64, x64, y64 = (t.astype(np.float64) for t in (A, x, y))
+    for pad, oa, ox, oy in FORMS:
+        Ap = np.full((M, N + pad), np.nan, np.float32)
+        Ap[:, :N] = A
+        bufs = [at(Ap, oa), at(x, ox)]
+        for beta in (0.5, 0.0):
+            out, py = at(y, oy)
+            L.lift_gemv_t(M, N, 1.25, bufs[0][1], N + pad, bufs[1][1], beta, py)
+            got = out[64 + oy:64 + oy + N].cpu().numpy().astype(np.float64)
+            ref = blas.gemv_t(A64, x64, y64, 1.25, beta)
+            terms = 1.25 * (np.abs(A64).T @ np.abs(x64)) + np.abs(beta * y64)
+            assert np.all(np.abs(got - ref) <= blas.tolerance(max(M, 2), 1.0) * terms), \
+                (pad, oa, ox, oy, beta)
+            assert torch.isnan(out[:64 + oy]).all() and torch.isnan(out[64 + oy + N:]).all()
