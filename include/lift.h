@@ -458,12 +458,12 @@ lift_status lift_features(int op, int64_t n, int64_t M, int64_t N, float* out);
  * lift_batch_create validates every descriptor (op id, variant id, sizes,
  * NULL or unaligned pointers) before touching the device and returns
  * LIFT_ERR_INVALID_ARG naming the first bad op; it then splits each op into
- * work items of about 256 KiB, orders the queue largest item first and
+ * work items of 64 to 256 KiB, orders the queue largest item first and
  * copies the descriptors to device memory it allocates (freed by
  * lift_batch_destroy).  Needs lift_init; call it outside stream capture.
  * lift_batch_run launches, on `stream`, a CUDA graph (captured on its first
- * call) made of a memset node that resets the queue head and the per-op
- * counters and the persistent kernel; the results are written when the
+ * call) made of the persistent kernel, which returns the queue head and the
+ * per-op counters to zero as it ends; the results are written when the
  * stream reaches the end of the graph.  Runs of one batch must not overlap.
  * Reduction results are the FP64 sum, rounded once, of per-item fp32
  * partials taken in item order, so they do not depend on scheduling.

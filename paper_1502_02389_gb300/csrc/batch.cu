@@ -12,12 +12,23 @@
 // each item leaves one fp32 partial, and the CTA that
 // finishes an op's last item (an atomic per-op counter) adds that op's item
 // partials in item order in FP64 (thread t takes partials t, t+256, ...,
-// then an FP64 block tree) and writes the rounded result.  Nothing waits:
-// the queue and the counters are atomics, reset by a memset node of the
-// same graph before the kernel node.  The other schedule of the same
-// map-workgroup launches one CTA per queue position instead of popping the
-// queue, and lets the hardware deal the CTAs to the SMs as earlier ones
+// then an FP64 block tree) and writes the rounded result; an op of one item
+// is written by the CTA that folds it.  Nothing waits: the queue and the
+// counters are atomics, and the CTAs that use them last return them to zero,
+// so that a run is one kernel and nothing else.  The other schedule of the
+// same map-workgroup launches one CTA per queue position instead of popping
+// the queue, and lets the hardware deal the CTAs to the SMs as earlier ones
 // retire; the items, their order and the combine are the same.
+//
+// A batch of small ops is bound by what a CTA does between items, so the
+// persistent kernel fetches ahead: while item i is folded, the first warp has
+// the op of item i+1, the item of i+2 and the queue position of i+3 in flight
+// (each CTA's first three positions are its own).  4000 ops of 2^8 to 2^14
+// elements and 64 to 256 rows and columns took 81 us when every item began
+// with the chain position -> item -> op -> data, ended with a fence and an
+// atomic, and the run began with two memset nodes; 48 now (22 at the copy
+// bandwidth).  Large batches are bound by DRAM: 2000 ops of 5.9 GB take
+// 861 us, the copy bandwidth's time (959 with gemv rows one at a time).
 //
 // Per op, the policy's variant choice (batch_pick: FIXED, TABLE or MLP) is
 // mapped to a processing mode: vector ops take the (tile, vector width) of
@@ -34,7 +45,12 @@ namespace lift {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int64_t kItemBytes = 256 * 1024;   // target bytes moved per work item
+// Bytes moved per work item: about 1/16 of a CTA's share of the batch, so
+// that the CTAs end together, but at least 64 KiB, so that an item is long
+// enough to hide the fetch of the next (118 ops of up to 4M elements: 68 us
+// with 64 KB items, 79 with 32 KB), and at most 256 KiB (2000 ops: 858 us
+// with 128 KB, 861 with 256 KB).
+constexpr int64_t kItemBytesMax = 256 * 1024, kItemBytesMin = 64 * 1024, kItemsPerCta = 16;
 
 // vector-op processing modes: (VW, J) with TILE = kThreads * VW * J
 struct VecMode {
@@ -57,17 +73,21 @@ struct OpDev {
 };
 
 struct ItemDev {
-  int op_index;
+  int op_index;         // -1: no item
+  int reserved;
+  int64_t index;        // of the item's partial: items of an op are consecutive
   int64_t begin, end;   // elements (vector ops) or rows (gemv)
 };
+constexpr int kOpChunks = sizeof(OpDev) / 16, kItemChunks = sizeof(ItemDev) / 16;
+static_assert(sizeof(OpDev) % 16 == 0 && sizeof(ItemDev) % 16 == 0 && kOpChunks + kItemChunks <= kWarp,
+              "a warp copies an op and an item in one go");
 
 struct BatchDev {
   const OpDev* ops;
-  const ItemDev* items;
-  const int64_t* order;       // queue position -> item index
-  float* partials;            // per item
-  unsigned* op_done;          // per op: items finished
-  unsigned long long* head;   // queue head
+  const ItemDev* items;       // in queue order
+  float* partials;            // per item index
+  unsigned* op_done;          // per op: items finished (0 between runs)
+  unsigned long long* head;   // queue positions dealt beyond the first, then CTAs that left (0 between runs)
   int64_t num_items;
 };
 
@@ -85,6 +105,8 @@ template <int OP, int VW, int J>
 __device__ float reduce_item(const OpDev& o, int64_t begin, int64_t end, float* red) {
   constexpr int64_t TILE = (int64_t)kThreads * VW * J;
   const int t = threadIdx.x;
+  const float* const x = o.x;
+  const float* const y = o.y;
   float acc = 0.f, cmp = 0.f;  // sum of the tile values and its Neumaier compensation
   int64_t base = begin;
   for (; base + TILE <= end; base += TILE) {
@@ -92,8 +114,8 @@ __device__ float reduce_item(const OpDev& o, int64_t begin, int64_t end, float* 
 #pragma unroll
     for (int j = 0; j < J; ++j) {
       const int64_t e = base + (int64_t)(t + kThreads * j) * VW;
-      ld_stream(o.x + e, a[j]);
-      if constexpr (OP == LIFT_OP_DOT) ld_stream(o.y + e, b[j]);
+      ld_stream(x + e, a[j]);
+      if constexpr (OP == LIFT_OP_DOT) ld_stream(y + e, b[j]);
     }
     float ts[VW];
 #pragma unroll
@@ -109,14 +131,20 @@ __device__ float reduce_item(const OpDev& o, int64_t begin, int64_t end, float* 
     float ts[VW];
 #pragma unroll
     for (int l = 0; l < VW; ++l) ts[l] = 0.f;
+    Vec<VW> a[J], b[J];                // all loads before the first fold
 #pragma unroll
     for (int j = 0; j < J; ++j) {
       const int64_t e = base + (int64_t)(t + kThreads * j) * VW;
-      Vec<VW> a, b;
-      ld_guarded<VW>(o.x, e, end, a);
-      if constexpr (OP == LIFT_OP_DOT) ld_guarded<VW>(o.y, e, end, b);
-      fold<OP, VW>(ts, a, b);
+      if (e + VW <= end) {
+        ld_stream(x + e, a[j]);
+        if constexpr (OP == LIFT_OP_DOT) ld_stream(y + e, b[j]);
+      } else {
+        ld_guarded<VW>(x, e, end, a[j]);
+        if constexpr (OP == LIFT_OP_DOT) ld_guarded<VW>(y, e, end, b[j]);
+      }
     }
+#pragma unroll
+    for (int j = 0; j < J; ++j) fold<OP, VW>(ts, a[j], b[j]);
     float tv = ts[0];
 #pragma unroll
     for (int l = 1; l < VW; ++l) tv = __fadd_rn(tv, ts[l]);
@@ -129,19 +157,43 @@ template <int VW, int J>
 __device__ void scal_item(const OpDev& o, int64_t begin, int64_t end) {
   constexpr int64_t TILE = (int64_t)kThreads * VW * J;
   const int t = threadIdx.x;
+  const float* const x = o.x;
+  float* const y = o.out;
+  const float alpha = o.alpha;
   int64_t base = begin;
   for (; base + TILE <= end; base += TILE) {
     Vec<VW> a[J];
 #pragma unroll
-    for (int j = 0; j < J; ++j) ld_stream(o.x + base + (int64_t)(t + kThreads * j) * VW, a[j]);
+    for (int j = 0; j < J; ++j) ld_stream(x + base + (int64_t)(t + kThreads * j) * VW, a[j]);
 #pragma unroll
     for (int j = 0; j < J; ++j) {
 #pragma unroll
-      for (int l = 0; l < VW; ++l) a[j].v[l] = __fmul_rn(o.alpha, a[j].v[l]);
-      st_stream(o.out + base + (int64_t)(t + kThreads * j) * VW, a[j]);
+      for (int l = 0; l < VW; ++l) a[j].v[l] = __fmul_rn(alpha, a[j].v[l]);
+      st_stream(y + base + (int64_t)(t + kThreads * j) * VW, a[j]);
     }
   }
-  for (int64_t e = base + t; e < end; e += kThreads) o.out[e] = __fmul_rn(o.alpha, o.x[e]);
+  if (base < end) {                    // the ragged tile: all loads before the first store
+    Vec<VW> a[J];
+#pragma unroll
+    for (int j = 0; j < J; ++j) {
+      const int64_t e = base + (int64_t)(t + kThreads * j) * VW;
+      if (e + VW <= end) ld_stream(x + e, a[j]);
+      else ld_guarded<VW>(x, e, end, a[j]);
+    }
+#pragma unroll
+    for (int j = 0; j < J; ++j) {
+      const int64_t e = base + (int64_t)(t + kThreads * j) * VW;
+#pragma unroll
+      for (int l = 0; l < VW; ++l) a[j].v[l] = __fmul_rn(alpha, a[j].v[l]);
+      if (e + VW <= end) {
+        st_stream(y + e, a[j]);
+      } else {
+#pragma unroll
+        for (int l = 0; l < VW; ++l)
+          if (e + l < end) y[e + l] = a[j].v[l];
+      }
+    }
+  }
 }
 
 template <int VW>
@@ -160,49 +212,78 @@ __device__ __forceinline__ void ld_x(const float* p, Vec<VW>& o) {
   }
 }
 
-template <int VW>
-__device__ void gemv_item(const OpDev& o, int64_t r0, int64_t r1) {
-  constexpr int64_t kChunk = (int64_t)kWarp * VW;
-  constexpr int U = VW == 1 ? 8 : (VW == 4 ? 4 : 2);
+// Rows [r0, r1) of op o, R consecutive rows per warp: a vector of x is loaded
+// once for R rows, and R * U vectors of A are in flight per lane.  Per row,
+// the arithmetic of the warp-per-row kernel.  Columns are counted in 32 bits
+// within pieces of 2^28 (whole groups), which keeps the loop in registers.
+template <int VW, int R, int U>
+__device__ __forceinline__ void gemv_item(const OpDev& o, int64_t r0, int64_t r1) {
+  constexpr int kStep = kWarp * VW, kPiece = 1 << 28;
+  static_assert(kGemvGroup % U == 0 && kPiece % (kGemvGroup * kStep) == 0, "whole groups");
   const int lane = threadIdx.x & (kWarp - 1);
-  const int64_t chunks = o.N / kChunk;
-  static_assert(kGemvGroup % U == 0, "an unrolled step stays inside one group");
-  for (int64_t row = r0 + threadIdx.x / kWarp; row < r1; row += kThreads / kWarp) {
-    const float* a = o.A + row * o.lda;
-    GroupedDot<VW> acc;
-    acc.init();
-    int64_t c = 0;                     // the lane's vector index along the row
-    for (; c + U <= chunks; c += U) {
-      Vec<VW> va[U], vx[U];
+  for (int64_t row = r0 + threadIdx.x / kWarp * R; row < r1; row += kThreads / kWarp * R) {
+    const int have = r1 - row < R ? (int)(r1 - row) : R;
+    float y0 = 0.f;                    // of row + lane, loaded ahead of the fold
+    if (o.beta != 0.f && lane < have) y0 = o.out[row + lane];
+    const float* a0 = o.A + row * o.lda + lane * VW;
+    const float* x = o.x + lane * VW;
+    GroupedDot<VW> acc[R];
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int64_t e = (c + u) * kChunk + lane * VW;
-        ld_stream(a + e, va[u]);
-        ld_x<VW>(o.x + e, vx[u]);
+    for (int r = 0; r < R; ++r) acc[r].init();
+    for (int64_t left = o.N; left > 0; left -= kPiece, a0 += kPiece, x += kPiece) {
+      const int n = (left < kPiece ? (int)left : kPiece) - lane * VW;   // columns from the lane's first
+      const float* a[R];
+#pragma unroll
+      for (int r = 0; r < R; ++r) a[r] = a0 + (r < have ? r : 0) * o.lda;
+      int c = 0, k = 0;                // k: the lane's vectors of the row (mod the group)
+      for (; c + (U - 1) * kStep + VW <= n; c += U * kStep) {
+        Vec<VW> va[R][U], vx[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+#pragma unroll
+          for (int r = 0; r < R; ++r) ld_stream(a[r] + c + u * kStep, va[r][u]);
+          ld_x<VW>(x + c + u * kStep, vx[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+          for (int r = 0; r < R; ++r) acc[r].add(va[r][u], vx[u]);
+        k = (k + U) & (kGemvGroup - 1);
+        if (k == 0) {
+#pragma unroll
+          for (int r = 0; r < R; ++r) acc[r].flush();
+        }
       }
+      if (c < n) {                     // the last, partial step: all its loads at once
+        Vec<VW> va[R][U], vx[U];
 #pragma unroll
-      for (int u = 0; u < U; ++u) acc.add(va[u], vx[u]);
-      if (((c + U) & (kGemvGroup - 1)) == 0) acc.flush();
+        for (int u = 0; u < U; ++u) {
+          const int e = c + u * kStep;
+          if (e + VW <= n) {
+#pragma unroll
+            for (int r = 0; r < R; ++r) ld_stream(a[r] + e, va[r][u]);
+            ld_x<VW>(x + e, vx[u]);
+          } else {
+#pragma unroll
+            for (int r = 0; r < R; ++r) ld_guarded<VW>(a[r], e, n, va[r][u]);
+            ld_guarded<VW>(x, e, n, vx[u]);
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+          for (int r = 0; r < R; ++r) acc[r].add(va[r][u], vx[u]);
+      }
     }
-    for (; c < chunks; ++c) {
-      Vec<VW> va, vx;
-      const int64_t e = c * kChunk + lane * VW;
-      ld_stream(a + e, va);
-      ld_x<VW>(o.x + e, vx);
-      acc.add(va, vx);
-      if (((c + 1) & (kGemvGroup - 1)) == 0) acc.flush();
+    float d = 0.f;                     // row + lane's dot
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const float v = __shfl_sync(0xffffffffu, warp_tree(acc[r].value()), 0);
+      if (lane == r) d = v;
     }
-    if (chunks * kChunk < o.N) {
-      Vec<VW> va, vx;
-      const int64_t e = chunks * kChunk + lane * VW;
-      ld_guarded<VW>(a, e, o.N, va);
-      ld_guarded<VW>(o.x, e, o.N, vx);
-      acc.add(va, vx);
-    }
-    float r = warp_tree(acc.value());
-    if (lane == 0) {
-      const float z = __fmul_rn(o.alpha, r);
-      o.out[row] = o.beta == 0.f ? z : __fadd_rn(z, __fmul_rn(o.beta, o.out[row]));
+    if (lane < have) {
+      const float z = __fmul_rn(o.alpha, d);
+      o.out[row + lane] = o.beta == 0.f ? z : __fadd_rn(z, __fmul_rn(o.beta, y0));
     }
   }
 }
@@ -219,6 +300,59 @@ __device__ float reduce_dispatch(const OpDev& o, int64_t b, int64_t e, float* re
   }
 }
 
+// One work item; `last` and the reduction scratch are shared by the CTA.
+__device__ __forceinline__ void run_item(const BatchDev& B, const ItemDev& item, const OpDev& o,
+                                         float* red, double* red64, bool* last) {
+  if (o.op == LIFT_OP_ASUM || o.op == LIFT_OP_DOT) {
+    const float r = o.op == LIFT_OP_ASUM ? reduce_dispatch<LIFT_OP_ASUM>(o, item.begin, item.end, red)
+                                         : reduce_dispatch<LIFT_OP_DOT>(o, item.begin, item.end, red);
+    if (o.num_items == 1) {            // the FP64 sum of one partial is the partial
+      if (threadIdx.x == 0) *o.out = __fadd_rn(0.f, r);
+      return;
+    }
+    if (threadIdx.x == 0) {
+      B.partials[item.index] = r;
+      __threadfence();
+      *last = atomicAdd(B.op_done + item.op_index, 1u) == (unsigned)(o.num_items - 1);
+    }
+    __syncthreads();
+    if (*last) {
+      __threadfence();
+      const double s = combine_partials<kThreads>(B.partials + o.first_item, o.num_items, red64);
+      if (threadIdx.x == 0) {
+        *o.out = static_cast<float>(s);
+        B.op_done[item.op_index] = 0u;   // ready for the next run
+      }
+    }
+  } else if (o.op == LIFT_OP_SCAL) {
+    switch (o.mode) {
+      case 0: scal_item<1, 4>(o, item.begin, item.end); break;
+      case 1: scal_item<4, 1>(o, item.begin, item.end); break;
+      case 2: scal_item<4, 2>(o, item.begin, item.end); break;
+      case 3: scal_item<4, 4>(o, item.begin, item.end); break;
+      case 4: scal_item<8, 1>(o, item.begin, item.end); break;
+      default: scal_item<8, 2>(o, item.begin, item.end); break;
+    }
+  } else {
+    switch (o.mode) {
+      case 0:
+        if (o.N <= 8 * kWarp) gemv_item<1, 4, 4>(o, item.begin, item.end);
+        else gemv_item<1, 2, 8>(o, item.begin, item.end);
+        break;
+      case 1:
+        if (item.end - item.begin > 16) gemv_item<4, 4, 1>(o, item.begin, item.end);
+        else gemv_item<4, 2, 2>(o, item.begin, item.end);
+        break;
+      default: gemv_item<8, 1, 2>(o, item.begin, item.end); break;
+    }
+  }
+}
+
+__device__ __forceinline__ void copy16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 // QUEUE: a persistent grid whose CTAs pop queue positions with an atomic;
 // otherwise one CTA per queue position (CTA q takes position q), dealt to
 // the SMs by the hardware in launch order as earlier CTAs retire.
@@ -226,70 +360,72 @@ template <bool QUEUE>
 __device__ __forceinline__ void batch_body(const BatchDev& B) {
   __shared__ float red[kWarp];
   __shared__ double red64[kWarp];
-  __shared__ int64_t s_item;
   __shared__ bool s_last;
-  for (;;) {
-    int64_t it;
-    if constexpr (QUEUE) {
-      if (threadIdx.x == 0) {
-        const unsigned long long q = atomicAdd(B.head, 1ull);
-        s_item = q < (unsigned long long)B.num_items ? B.order[q] : -1;
+  if constexpr (!QUEUE) {
+    if ((int64_t)blockIdx.x >= B.num_items) return;
+    const ItemDev item = B.items[blockIdx.x];
+    run_item(B, item, B.ops[item.op_index], red, red64, &s_last);
+  } else {
+    __shared__ __align__(16) ItemDev s_item[3];     // items i, i + 1 and the slot of i + 2
+    __shared__ __align__(16) OpDev s_op[2];         // their ops, i and i + 1
+    const int lane = threadIdx.x & (kWarp - 1);
+    const bool fetcher = threadIdx.x < kWarp;
+    const unsigned long long G = gridDim.x;
+    // start the copy of the item at queue position q (op_index -1 past the
+    // end), and of an op; lanes 0.. and kOpChunks.. move 16 bytes each
+    auto get_item = [&](int slot, unsigned long long q) {
+      const int k = lane - kOpChunks;
+      if (q >= (unsigned long long)B.num_items) {
+        if (k == 0) s_item[slot].op_index = -1;
+      } else if (k >= 0 && k < kItemChunks) {
+        copy16(reinterpret_cast<char*>(s_item + slot) + 16 * k,
+               reinterpret_cast<const char*>(B.items + q) + 16 * k);
       }
-      __syncthreads();
-      it = s_item;
-    } else {
-      it = (int64_t)blockIdx.x < B.num_items ? B.order[blockIdx.x] : -1;
+    };
+    auto get_op = [&](int slot, int op) {
+      if (op >= 0 && lane < kOpChunks)
+        copy16(reinterpret_cast<char*>(s_op + slot) + 16 * lane,
+               reinterpret_cast<const char*>(B.ops + op) + 16 * lane);
+    };
+    unsigned long long q = 0;                       // queue position of item i + 2 (lane 0's)
+    if (fetcher) {
+      get_item(0, blockIdx.x);
+      get_item(1, blockIdx.x + G);
+      q = blockIdx.x + 2 * G;
+      copy_wait();
+      __syncwarp();
+      get_op(0, s_item[0].op_index);
+      copy_wait();
     }
-    if (it < 0) return;
-    const ItemDev item = B.items[it];
-    const OpDev o = B.ops[item.op_index];
-    if (o.op == LIFT_OP_ASUM || o.op == LIFT_OP_DOT) {
-      const float r = o.op == LIFT_OP_ASUM ? reduce_dispatch<LIFT_OP_ASUM>(o, item.begin, item.end, red)
-                                           : reduce_dispatch<LIFT_OP_DOT>(o, item.begin, item.end, red);
-      if (threadIdx.x == 0) {
-        B.partials[it] = r;
+    __syncthreads();
+    for (int i = 0, i3 = 0; s_item[i3].op_index >= 0; i ^= 1, i3 = i3 == 2 ? 0 : i3 + 1) {
+      if (fetcher) {
+        get_op(i ^ 1, s_item[i3 == 2 ? 0 : i3 + 1].op_index);
+        get_item(i3 == 0 ? 2 : i3 - 1, __shfl_sync(0xffffffffu, q, 0));
+        if (lane == 0) q = atomicAdd(B.head, 1ull) + 3 * G;
+      }
+      run_item(B, s_item[i3], s_op[i], red, red64, &s_last);
+      if (fetcher) copy_wait();
+      __syncthreads();   // shared state is reused by the next item
+    }
+    // the last CTA to leave returns the queue to its start
+    if (threadIdx.x == 0) {
+      __threadfence();
+      if (atomicAdd(B.head + 1, 1ull) == G - 1) {
         __threadfence();
-        s_last = atomicAdd(B.op_done + item.op_index, 1u) == (unsigned)(o.num_items - 1);
-      }
-      __syncthreads();
-      if (s_last) {
-        __threadfence();
-        const double s = combine_partials<kThreads>(B.partials + o.first_item, o.num_items, red64);
-        if (threadIdx.x == 0) *o.out = static_cast<float>(s);
-      }
-    } else if (o.op == LIFT_OP_SCAL) {
-      switch (o.mode) {
-        case 0: scal_item<1, 4>(o, item.begin, item.end); break;
-        case 1: scal_item<4, 1>(o, item.begin, item.end); break;
-        case 2: scal_item<4, 2>(o, item.begin, item.end); break;
-        case 3: scal_item<4, 4>(o, item.begin, item.end); break;
-        case 4: scal_item<8, 1>(o, item.begin, item.end); break;
-        default: scal_item<8, 2>(o, item.begin, item.end); break;
-      }
-    } else {
-      switch (o.mode) {
-        case 0: gemv_item<1>(o, item.begin, item.end); break;
-        case 1: gemv_item<4>(o, item.begin, item.end); break;
-        default: gemv_item<8>(o, item.begin, item.end); break;
+        B.head[0] = 0ull;
+        B.head[1] = 0ull;
       }
     }
-    if constexpr (!QUEUE) return;
-    __syncthreads();   // shared state is reused by the next item
   }
 }
 
-// The kernels: batches of vector ops leave the register allocation to the
-// compiler (64 registers, 4 CTAs per SM); batches with gemv ops ask for 5
-// CTAs per SM (48 registers): their warp-per-row items keep more rows in
-// flight with the extra warps (the 20,000-op workload: 8.89 ms against
-// 9.44 ms), while vector ops alone ran about 1 % slower that way.
+// 4 CTAs per SM (64 registers).  With the rows of gemv items loaded one at a
+// time a batch with gemv ops wanted 5 (48 registers); several rows per warp
+// have more loads in flight on fewer warps, and spill at 48 (2000 ops: 887 us
+// against 866).
 template <bool QUEUE>
-__global__ void __launch_bounds__(kThreads) batch_kernel(BatchDev B) {
-  batch_body<QUEUE>(B);
-}
-
-template <bool QUEUE>
-__global__ void __launch_bounds__(kThreads, 5) batch_kernel_gemv(BatchDev B) {
+__global__ void __launch_bounds__(kThreads, 4) batch_kernel(BatchDev B) {
   batch_body<QUEUE>(B);
 }
 
@@ -305,13 +441,11 @@ struct lift_batch {
   std::vector<int64_t> item;  // per op: elements (or rows) per work item
   lift::OpDev* ops = nullptr;
   lift::ItemDev* items = nullptr;
-  int64_t* order = nullptr;
   float* partials = nullptr;
   unsigned* op_done = nullptr;
   unsigned long long* head = nullptr;
   int64_t grid = 0;           // CTAs of the persistent (queue) grid
   int schedule = LIFT_BATCH_QUEUE;
-  bool gemv_occupancy = false;  // a gemv op is present: the 5-CTAs-per-SM kernel
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
 };
@@ -334,7 +468,6 @@ void free_batch(lift_batch* b) {
   if (b->graph) cudaGraphDestroy(b->graph);
   cudaFree(b->ops);
   cudaFree(b->items);
-  cudaFree(b->order);
   cudaFree(b->partials);
   cudaFree(b->op_done);
   cudaFree(b->head);
@@ -391,6 +524,19 @@ lift_status lift_batch_create(const lift_op_desc* descs, int64_t count, lift_bat
   b->item.resize(count);
   std::vector<ItemDev> items;
   std::vector<std::pair<int64_t, int64_t>> cost;   // (bytes, item) for the queue order
+  int per_sm = 0;
+  lift_status rc = cuda_check(
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel<true>, kThreads, 0),
+      "batch occupancy");
+  if (rc != LIFT_OK) {
+    delete b;
+    return rc;
+  }
+  b->grid = (int64_t)per_sm * st->sm_count;
+  int64_t total = 0;
+  for (int64_t i = 0; i < count; ++i) total += op_bytes(descs[i]);
+  const int64_t item_bytes = std::min(
+      kItemBytesMax, std::max(kItemBytesMin, total / (std::max<int64_t>(1, b->grid) * kItemsPerCta)));
   for (int64_t i = 0; i < count; ++i) {
     const lift_op_desc& d = descs[i];
     OpDev o{};
@@ -416,12 +562,12 @@ lift_status lift_batch_create(const lift_op_desc* descs, int64_t count, lift_bat
       if (!aligned(d.A, 4 * vw) || !aligned(d.x, 4 * vw) || (d.lda * 4) % (4 * vw) != 0) m = 0;
       o.mode = m;
       const int64_t row_bytes = 4 * (d.N > 0 ? d.N : 1);
-      int64_t rows = std::max<int64_t>(8, kItemBytes / row_bytes / 8 * 8);
+      int64_t rows = std::max<int64_t>(16, item_bytes / row_bytes / 16 * 16);
       b->item[i] = rows;
       for (int64_t r = 0; r < d.M; r += rows) {
         const int64_t e = std::min(d.M, r + rows);
         cost.push_back({(e - r) * row_bytes, (int64_t)items.size()});
-        items.push_back({(int)i, r, e});
+        items.push_back({(int)i, 0, (int64_t)items.size(), r, e});
       }
     } else {
       int m = vec_mode_for(info);
@@ -432,16 +578,16 @@ lift_status lift_batch_create(const lift_op_desc* descs, int64_t count, lift_bat
       o.mode = m;
       const int64_t tile = (int64_t)kThreads * kVecModes[m].vw * kVecModes[m].j;
       const int64_t esz = d.op == LIFT_OP_ASUM ? 4 : 8;
-      const int64_t per = std::max<int64_t>(1, kItemBytes / (tile * esz)) * tile;
+      const int64_t per = std::max<int64_t>(1, item_bytes / (tile * esz)) * tile;
       b->item[i] = per;
       if (d.n == 0 && d.op != LIFT_OP_SCAL) {
         cost.push_back({0, (int64_t)items.size()});
-        items.push_back({(int)i, 0, 0});   // one empty item: the combine writes 0
+        items.push_back({(int)i, 0, (int64_t)items.size(), 0, 0});   // one empty item: the combine writes 0
       }
       for (int64_t s = 0; s < d.n; s += per) {
         const int64_t e = std::min(d.n, s + per);
         cost.push_back({(e - s) * esz, (int64_t)items.size()});
-        items.push_back({(int)i, s, e});
+        items.push_back({(int)i, 0, (int64_t)items.size(), s, e});
       }
     }
     o.num_items = (int64_t)items.size() - o.first_item;
@@ -454,36 +600,25 @@ lift_status lift_batch_create(const lift_op_desc* descs, int64_t count, lift_bat
                    [](const std::pair<int64_t, int64_t>& a, const std::pair<int64_t, int64_t>& c) {
                      return a.first > c.first;
                    });
-  std::vector<int64_t> order(items.size());
-  for (size_t k = 0; k < cost.size(); ++k) order[k] = cost[k].second;
+  std::vector<ItemDev> queue(items.size());
+  for (size_t k = 0; k < cost.size(); ++k) queue[k] = items[cost[k].second];
+  if (b->grid > b->num_items) b->grid = std::max<int64_t>(1, b->num_items);
 
   const size_t ni = std::max<size_t>(1, items.size()), no = std::max<int64_t>(1, count);
-  lift_status rc = cuda_check(cudaMalloc(&b->ops, no * sizeof(OpDev)), "batch alloc");
+  rc = cuda_check(cudaMalloc(&b->ops, no * sizeof(OpDev)), "batch alloc");
   if (rc == LIFT_OK) rc = cuda_check(cudaMalloc(&b->items, ni * sizeof(ItemDev)), "batch alloc");
-  if (rc == LIFT_OK) rc = cuda_check(cudaMalloc(&b->order, ni * sizeof(int64_t)), "batch alloc");
   if (rc == LIFT_OK) rc = cuda_check(cudaMalloc(&b->partials, ni * sizeof(float)), "batch alloc");
   if (rc == LIFT_OK) rc = cuda_check(cudaMalloc(&b->op_done, no * sizeof(unsigned)), "batch alloc");
-  if (rc == LIFT_OK) rc = cuda_check(cudaMalloc(&b->head, sizeof(unsigned long long)), "batch alloc");
+  if (rc == LIFT_OK) rc = cuda_check(cudaMalloc(&b->head, 2 * sizeof(unsigned long long)), "batch alloc");
+  if (rc == LIFT_OK) rc = cuda_check(cudaMemset(b->op_done, 0, no * sizeof(unsigned)), "batch init");
+  if (rc == LIFT_OK)
+    rc = cuda_check(cudaMemset(b->head, 0, 2 * sizeof(unsigned long long)), "batch init");
   if (rc == LIFT_OK && count > 0)
     rc = cuda_check(cudaMemcpy(b->ops, b->ops_host.data(), count * sizeof(OpDev), cudaMemcpyHostToDevice),
                     "batch upload");
   if (rc == LIFT_OK && !items.empty())
-    rc = cuda_check(cudaMemcpy(b->items, items.data(), items.size() * sizeof(ItemDev),
+    rc = cuda_check(cudaMemcpy(b->items, queue.data(), queue.size() * sizeof(ItemDev),
                                cudaMemcpyHostToDevice), "batch upload");
-  if (rc == LIFT_OK && !items.empty())
-    rc = cuda_check(cudaMemcpy(b->order, order.data(), order.size() * sizeof(int64_t),
-                               cudaMemcpyHostToDevice), "batch upload");
-  if (rc == LIFT_OK) {
-    int per_sm = 0;
-    b->gemv_occupancy = std::any_of(b->ops_host.begin(), b->ops_host.end(),
-                                    [](const OpDev& o) { return o.op == LIFT_OP_GEMV; });
-    rc = cuda_check(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                        &per_sm, b->gemv_occupancy ? batch_kernel_gemv<true> : batch_kernel<true>,
-                        kThreads, 0),
-                    "batch occupancy");
-    b->grid = (int64_t)per_sm * st->sm_count;
-    if (b->grid > b->num_items) b->grid = std::max<int64_t>(1, b->num_items);
-  }
   if (rc != LIFT_OK) {
     free_batch(b);
     return rc;
@@ -492,8 +627,8 @@ lift_status lift_batch_create(const lift_op_desc* descs, int64_t count, lift_bat
   return LIFT_OK;
 }
 
-// The graph: memset(head, op counters) -> batch_kernel, captured once on a
-// private stream, then launched on the caller's stream.
+// The graph: batch_kernel, captured once on a private stream, then launched
+// on the caller's stream.
 lift_status lift_batch_run(lift_batch* b, void* stream) {
   if (!b) return set_error(LIFT_ERR_INVALID_ARG, "batch is NULL");
   if (b->num_items == 0) return LIFT_OK;
@@ -503,14 +638,10 @@ lift_status lift_batch_run(lift_batch* b, void* stream) {
     if (rc != LIFT_OK) return rc;
     rc = cuda_check(cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal), "capture");
     if (rc == LIFT_OK) {
-      cudaMemsetAsync(b->head, 0, sizeof(unsigned long long), cap);
-      cudaMemsetAsync(b->op_done, 0, std::max<int64_t>(1, b->count) * sizeof(unsigned), cap);
-      BatchDev B{b->ops, b->items, b->order, b->partials, b->op_done, b->head, b->num_items};
+      BatchDev B{b->ops, b->items, b->partials, b->op_done, b->head, b->num_items};
       const bool q = b->schedule == LIFT_BATCH_QUEUE;
       const unsigned g = (unsigned)(q ? b->grid : b->num_items);
-      if (q && b->gemv_occupancy) batch_kernel_gemv<true><<<g, kThreads, 0, cap>>>(B);
-      else if (q) batch_kernel<true><<<g, kThreads, 0, cap>>>(B);
-      else if (b->gemv_occupancy) batch_kernel_gemv<false><<<g, kThreads, 0, cap>>>(B);
+      if (q) batch_kernel<true><<<g, kThreads, 0, cap>>>(B);
       else batch_kernel<false><<<g, kThreads, 0, cap>>>(B);
       rc = cuda_check(cudaStreamEndCapture(cap, &b->graph), "end capture");
     }
