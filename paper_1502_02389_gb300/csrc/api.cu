@@ -154,6 +154,7 @@ void register_gemv_pertile(std::vector<Variant>& gemv);  // scal_gemv.cu (one CT
 void register_blackscholes(std::vector<Variant>& bs);  // blackscholes.cu
 void register_compensated(std::vector<Variant>& asum, std::vector<Variant>& dot);  // compensated.cu
 void register_reduce_derived(std::vector<Variant>& asum, std::vector<Variant>& dot);  // reduce_derived.cu
+const Variant* unaligned_form(int op);   // unaligned.cu
 void gemv_split_shape(int k, const Args& a, int64_t* L, int64_t* S);
 void register_gemv_rows(std::vector<Variant>& gemv);   // gemv_rows.cu (several rows at a time)
 void gemv_split_rows_shape(const char* name, const Args& a, int64_t* L, int64_t* S);
@@ -745,17 +746,29 @@ int batch_pick(int op, int64_t n, int64_t M, int64_t N) {
   return pick_variant(op, a, nullptr, false, false);
 }
 
-// Resolve the variant to run: explicit id or policy pick, then the guarded
-// form when a pointer is not aligned for the chosen variant.
+static bool overridden(int op) {
+  std::lock_guard<std::mutex> lk(g_policy_mu);
+  return g_override[op] >= 0;
+}
+
+// Resolve the variant to run: explicit id or policy pick.  When a pointer is
+// not aligned for it, a variant asked for by id (here or with
+// lift_set_variant) runs its guarded form, and the policy's own pick the
+// op's unaligned form where there is one.
 static lift_status resolve(int op, int variant, const Args& a, const Variant** out,
                            cudaStream_t s = nullptr, bool may_tune = false) {
   auto& L = registry(op);
   if (L.empty()) return set_error(LIFT_ERR_UNSUPPORTED, "no variants for op");
   if (variant < -1 || variant >= (int)L.size())
     return set_error(LIFT_ERR_INVALID_ARG, "variant id out of range");
-  if (variant < 0) variant = pick_variant(op, a, s, may_tune);
+  const bool picked = variant < 0;
+  if (picked) variant = pick_variant(op, a, s, may_tune);
   const Variant* v = &L[variant];
-  if (!eligible(op, *v, a) && v->fallback >= 0) v = &L[v->fallback];
+  if (!eligible(op, *v, a)) {
+    const Variant* u = picked && !overridden(op) ? unaligned_form(op) : nullptr;
+    if (u) v = u;
+    else if (v->fallback >= 0) v = &L[v->fallback];
+  }
   *out = v;
   return LIFT_OK;
 }

@@ -83,3 +83,51 @@ def test_gemv_t(L, M, N):
             assert np.all(np.abs(got - ref) <= blas.tolerance(max(M, 2), 1.0) * terms), \
                 (pad, oa, ox, oy, beta)
             assert torch.isnan(out[:64 + oy]).all() and torch.isnan(out[64 + oy + N:]).all()
+
+
+# the default vector entry points on slices: every pair of offsets, sizes
+# around the vectors and tiles (2048 elements for the maps, 4096 for the
+# reductions), NaN on both sides of every array
+@pytest.mark.parametrize("n", [1, 2, 3, 5, 31, 2045, 2048, 4093, 4096, 4099, 8195, 20001, 1300001])
+def test_unaligned_vectors(L, n):
+    rng = np.random.default_rng(n)
+    x, y = rng.standard_normal(n).astype(np.float32), rng.standard_normal(n).astype(np.float32)
+    x64, y64 = x.astype(np.float64), y.astype(np.float64)
+    scal = (x64 * 1.5).astype(np.float32)
+    axpy = (np.float32(-0.75) * x + y).astype(np.float32)      # fl(fl(a x) + y): two roundings
+    nrm = float(np.sqrt(np.sum(x64 * x64)))
+    want = [(L.lift_asum, blas.asum(x64), blas.asum_terms(x)), (L.lift_asum_comp, blas.asum(x64), None),
+            (L.lift_sum, float(np.sum(x64)), blas.asum_terms(x)), (L.lift_nrm2, nrm, nrm)]
+    for ox in range(4):
+        bx, px = at(x, ox)
+        for f, ref, terms in want:
+            r = torch.full((1,), -7.0, device="cuda")
+            f(px, n, r)
+            tol = blas.tolerance(max(2, n), terms) if terms is not None else 2.0 ** -22 * abs(ref)
+            assert abs(float(r.item()) - ref) <= tol, (f.__name__, ox)
+        for oy in range(4):
+            by, py = at(y, oy)
+            r = torch.full((2,), -7.0, device="cuda")
+            L.lift_dot(px, py, n, r[0:1])
+            L.lift_dot_comp(px, py, n, r[1:2])
+            ref, terms = blas.dot(x64, y64), blas.dot_terms(x, y)
+            got = r.cpu().numpy().astype(np.float64)
+            assert np.all(np.abs(got - ref) <= blas.tolerance(max(2, n), terms)), (ox, oy)
+            L.lift_axpy(n, -0.75, px, py)
+            assert np.array_equal(by[64 + oy:64 + oy + n].cpu().numpy().view(np.uint32),
+                                  axpy.view(np.uint32)), (ox, oy)
+            L.lift_scal(n, 1.5, px, py)
+            assert np.array_equal(by[64 + oy:64 + oy + n].cpu().numpy().view(np.uint32),
+                                  scal.view(np.uint32)), (ox, oy)
+            assert torch.isnan(by[:64 + oy]).all() and torch.isnan(by[64 + oy + n:]).all()
+        L.lift_scal(n, 1.5, px, px)                            # in place
+        assert np.array_equal(bx[64 + ox:64 + ox + n].cpu().numpy().view(np.uint32),
+                              scal.view(np.uint32)), ox
+        assert torch.isnan(bx[:64 + ox]).all() and torch.isnan(bx[64 + ox + n:]).all()
+    v = torch.ones(n + 8, device="cuda")                       # Inf and NaN propagate
+    v[1 + n // 2] = float("inf")
+    r = torch.zeros(1, device="cuda")
+    L.lift_asum(v.data_ptr() + 4, n, r)
+    assert r.item() == float("inf")
+    L.lift_asum(v.data_ptr() + 8, 0, r)                        # an empty slice
+    assert r.item() == 0.0
