@@ -130,6 +130,11 @@ template <int THREADS, int VW, int U, int CND>
 __global__ void __launch_bounds__(THREADS)
     bs_map(int64_t n, const float* __restrict__ s, float* __restrict__ call,
            float* __restrict__ put, BsConst c) {
+  if (threadIdx.x == 0 && blockIdx.x < kPrefetchCtas) {
+    constexpr int kPer = THREADS * U * VW;
+    const int64_t e = own(blockIdx.x) * kPer;
+    if (e + kPer <= own(n)) prefetch_l2(s + e, kPer * sizeof(float));
+  }
   pdl_trigger();   // the next call's first kernel may be scheduled (it waits for this one)
   pdl_wait();      // the previous kernel on the stream has completed
   const int64_t nv = n / VW;                         // whole vectors

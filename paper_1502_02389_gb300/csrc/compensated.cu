@@ -41,6 +41,15 @@ __global__ void __launch_bounds__(THREADS)
     comp_reduce(const float* __restrict__ x, const float* __restrict__ y, int64_t n,
                 double* __restrict__ partials, unsigned* ticket, float* result, double* result64) {
   constexpr int64_t kTile = (int64_t)THREADS * VW * U;
+  // the CTA's first two tiles, in calls of up to 16 tiles per CTA (dot, n =
+  // 2^24: 24.3 -> 23.2 us; n = 2^26 would take 80.1 with it, 78.7 without)
+  if (threadIdx.x < 2) {
+    const int64_t tiles = own(n) / kTile, p = own(blockIdx.x) + threadIdx.x * (int64_t)gridDim.x;
+    if (tiles < 16 * (int64_t)gridDim.x && p < tiles) {
+      prefetch_l2(x + p * kTile, kTile * sizeof(float));
+      if constexpr (OP == LIFT_OP_DOT) prefetch_l2(y + p * kTile, kTile * sizeof(float));
+    }
+  }
   pdl_wait();      // the previous kernel on the stream has completed
   const int t = threadIdx.x;
   const int64_t G = gridDim.x;

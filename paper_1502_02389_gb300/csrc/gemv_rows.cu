@@ -115,10 +115,14 @@ __global__ void __launch_bounds__(THREADS)
   constexpr int W = THREADS / kWarp;
   static_assert(R <= W, "one warp per row in the last stage of the tree");
   __shared__ float red[R][kWarp];
-  pdl_wait();      // the previous kernel on the stream has completed
   const int lane = threadIdx.x & (kWarp - 1), warp = threadIdx.x / kWarp;
   const int64_t r0 = blockIdx.x / S * R, seg = blockIdx.x % S;
   const int64_t c_end = (seg + 1) * L < N ? (seg + 1) * L : N;
+  if (threadIdx.x < R && blockIdx.x < kPrefetchCtas && r0 + threadIdx.x < M) {   // two steps of every row
+    const int64_t c = seg * L, len = c_end - c < 2 * U * THREADS * VW ? c_end - c : 2 * U * THREADS * VW;
+    prefetch_l2(A + (r0 + threadIdx.x) * lda + c, 4 * len);
+  }
+  pdl_wait();      // the previous kernel on the stream has completed
   const float* a[R];
   row_pointers<R>(A, lda, r0, M, a);
   GroupedDot<VW> acc[R];
@@ -148,10 +152,13 @@ template <int WARPS, int VW, int R, int U>
 __global__ void __launch_bounds__(WARPS * kWarp)
     gemv_warp_rows(int64_t M, int64_t N, float alpha, const float* __restrict__ A, int64_t lda,
                    const float* __restrict__ x, float beta, float* __restrict__ y) {
-  pdl_trigger();   // the next call's first kernel may be scheduled (it waits for this one)
-  pdl_wait();      // the previous kernel on the stream has completed
   const int lane = threadIdx.x & (kWarp - 1);
   const int64_t total = (int64_t)gridDim.x * WARPS * R;
+  const int64_t first = ((int64_t)blockIdx.x * WARPS + threadIdx.x / kWarp) * R + lane;
+  if (lane < R && blockIdx.x < kPrefetchCtas && first < M)
+    prefetch_l2(A + first * lda, 4 * (N < 2048 ? N : 2048));
+  pdl_trigger();   // the next call's first kernel may be scheduled (it waits for this one)
+  pdl_wait();      // the previous kernel on the stream has completed
   for (int64_t r0 = ((int64_t)blockIdx.x * WARPS + threadIdx.x / kWarp) * R; r0 < M; r0 += total) {
     const float* a[R];
     row_pointers<R>(A, lda, r0, M, a);

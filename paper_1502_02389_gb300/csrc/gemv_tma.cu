@@ -66,6 +66,10 @@ __global__ void __launch_bounds__((WARPS + 1) * kWarp, 1)
     }
     fence_mbar_init();
   }
+  if (warp == WARPS && lane < WARPS && r_begin + lane < r_end) {   // the first ring of the first rows
+    const int64_t len = N < (int64_t)S * C ? N : (int64_t)S * C;
+    prefetch_l2(A + (r_begin + lane) * lda, 4 * len);
+  }
   pdl_trigger();   // the next call's first kernel may be scheduled (it waits for this one)
   pdl_wait();      // the previous kernel on the stream has completed
   __syncthreads();

@@ -43,11 +43,23 @@ __device__ __forceinline__ void scal_tail(int64_t n, float alpha, const float* x
   }
 }
 
-template <int THREADS, int TILE, int VW>
+// AHEAD: the first wave of CTAs asks for its tiles before the previous call
+// has ended; for calls of up to kAheadTiles tiles (2048-element tiles in a
+// graph of calls: n = 2^20 3.0 -> 2.3 us, n = 2^22 6.6 -> 6.0).  In longer
+// calls it gains nothing, and the kernel that holds it takes three registers
+// less, eight CTAs per SM instead of seven, and then 77.2 us at n = 2^26
+// instead of 75.4: the map's two streams want fewer CTAs.
+constexpr int64_t kAheadTiles = 4096;
+
+template <int THREADS, int TILE, int VW, bool AHEAD>
 __global__ void __launch_bounds__(THREADS)
     scal_ldg(int64_t n, float alpha, const float* x, float* y) {
   constexpr int J = TILE / VW / THREADS;
   static_assert(J >= 1 && (TILE / VW) % THREADS == 0, "tile too small");
+  if constexpr (AHEAD) {
+    if (threadIdx.x == 0 && blockIdx.x < kPrefetchCtas && ((int64_t)blockIdx.x + 1) * TILE <= n)
+      prefetch_l2(x + (int64_t)blockIdx.x * TILE, TILE * sizeof(float));
+  }
   pdl_trigger();   // the next call's first kernel may be scheduled (it waits for this one)
   pdl_wait();      // the previous kernel on the stream has completed
   const int64_t full = n / TILE;
@@ -148,7 +160,7 @@ struct Scal {
   static_assert(GRID == 0 || STAGES == 0, "a staged ring needs several tiles per CTA");
   static const void* kernel() {
     if constexpr (STAGES == 0)
-      return reinterpret_cast<const void*>(&scal_ldg<THREADS, TILE, VW>);
+      return reinterpret_cast<const void*>(&scal_ldg<THREADS, TILE, VW, false>);
     else
       return reinterpret_cast<const void*>(&scal_tma<THREADS, TILE, STAGES>);
   }
@@ -167,6 +179,10 @@ struct Scal {
     int* status = current_state()->ws.status;
     if constexpr (STAGES == 0) {
       void* args[] = {&n, &alpha, &x, &y};
+      if (n <= kAheadTiles * TILE) {
+        const void* ahead = reinterpret_cast<const void*>(&scal_ldg<THREADS, TILE, VW, true>);
+        return launch_config(ahead, dim3((unsigned)g), dim3(THREADS), 0, 1, s, args, true);
+      }
       return launch_config(kernel(), dim3((unsigned)g), dim3(THREADS), 0, 1, s, args, true);
     } else {
       void* args[] = {&n, &alpha, &x, &y, &status};
@@ -206,6 +222,10 @@ __global__ void __launch_bounds__(THREADS)
     axpy_ldg(int64_t n, float alpha, const float* x, float* y) {
   constexpr int J = TILE / VW / THREADS;
   static_assert(J >= 1 && (TILE / VW) % THREADS == 0, "tile too small");
+  if (threadIdx.x < 2 && blockIdx.x < kPrefetchCtas) {
+    const int64_t p = own(blockIdx.x);
+    if ((p + 1) * TILE <= n) prefetch_l2((threadIdx.x == 0 ? x : y) + p * TILE, TILE * sizeof(float));
+  }
   pdl_trigger();   // the next call's first kernel may be scheduled (it waits for this one)
   pdl_wait();      // the previous kernel on the stream has completed
   const int64_t full = n / TILE;

@@ -140,9 +140,14 @@ __global__ void __launch_bounds__(kUnThreads)
   __shared__ float red[kWarp];
   __shared__ double red64[kWarp];
   __shared__ bool is_last;
-  pdl_wait();      // the previous kernel on the stream has completed
   const int t = threadIdx.x, lane = t & (kWarp - 1);
   const int64_t G = gridDim.x, T = (hi + kUnTile - 1) / kUnTile;
+  if (t < 2 && whole_tile(blockIdx.x + t * G, kUnTile, lo, hi, d)) {    // the CTA's first two tiles
+    const int64_t e = (blockIdx.x + t * G) * kUnTile;
+    prefetch_l2(x + e, kUnTile * sizeof(float));
+    if constexpr (F::kTwo) prefetch_l2(y + e, kUnTile * sizeof(float));
+  }
+  pdl_wait();      // the previous kernel on the stream has completed
   const int64_t off = (int64_t)(t / kWarp) * (kWarp * 4 * J);     // the warp's part of a tile
   F f;
   Vec<4> cx[J + 1], cy[J + 1];
@@ -213,10 +218,12 @@ template <bool AXPY>
 __global__ void __launch_bounds__(kUnThreads)
     unaligned_map(const float* x, float* y, int64_t lo, int64_t hi, int d, float alpha) {
   constexpr int J = kMapVecs;
-  pdl_trigger();   // the next call's first kernel may be scheduled (it waits for this one)
-  pdl_wait();      // the previous kernel on the stream has completed
   const int lane = threadIdx.x & (kWarp - 1);
   const int64_t tile = blockIdx.x;
+  if (threadIdx.x < (AXPY ? 2 : 1) && tile < kPrefetchCtas && whole_tile(tile, kMapTile, lo, hi, d))
+    prefetch_l2((threadIdx.x == 0 ? x : y) + tile * kMapTile, kMapTile * sizeof(float));
+  pdl_trigger();   // the next call's first kernel may be scheduled (it waits for this one)
+  pdl_wait();      // the previous kernel on the stream has completed
   const int64_t e = tile * kMapTile + (int64_t)(threadIdx.x / kWarp) * (kWarp * 4 * J);
   const bool whole = whole_tile(tile, kMapTile, lo, hi, d);
   Vec<4> a[J + 1], b[J];
