@@ -219,8 +219,8 @@ __global__ void __launch_bounds__(kUnThreads)
     unaligned_map(const float* x, float* y, int64_t lo, int64_t hi, int d, float alpha) {
   constexpr int J = kMapVecs;
   const int lane = threadIdx.x & (kWarp - 1);
-  const int64_t tile = blockIdx.x;
-  if (threadIdx.x < (AXPY ? 2 : 1) && tile < kPrefetchCtas && whole_tile(tile, kMapTile, lo, hi, d))
+  const int64_t tile = gridDim.x - 1 - blockIdx.x;          // last tile first
+  if (threadIdx.x < (AXPY ? 2 : 1) && blockIdx.x < kPrefetchCtas && whole_tile(tile, kMapTile, lo, hi, d))
     prefetch_l2((threadIdx.x == 0 ? x : y) + tile * kMapTile, kMapTile * sizeof(float));
   pdl_trigger();   // the next call's first kernel may be scheduled (it waits for this one)
   pdl_wait();      // the previous kernel on the stream has completed
