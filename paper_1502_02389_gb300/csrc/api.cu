@@ -46,9 +46,15 @@ constexpr int64_t kPartialCapacity = 1 << 22;   // fp32 partial slots per worksp
 constexpr int64_t kPartial64Capacity = 1 << 17; // FP64 partial slots per workspace slot (1 MiB)
 extern const int kTicketSlots = 64 + 65536;     // counters: reductions, then gemv-T column blocks
 
+// The states again, by device ordinal, for current_state: every call asks
+// several times, and a map behind a mutex showed in the submission time.
+constexpr int kFastDevices = 64;
+static std::atomic<DeviceState*> g_fast[kFastDevices];
+
 DeviceState* current_state() {
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
+  if (dev >= 0 && dev < kFastDevices) return g_fast[dev].load(std::memory_order_acquire);
   std::lock_guard<std::mutex> lk(g_mu);
   auto it = g_states.find(dev);
   return it == g_states.end() ? nullptr : it->second;
@@ -132,6 +138,7 @@ static lift_status init_device(int device) {
   {
     std::lock_guard<std::mutex> lk(g_mu);
     g_states[device] = st;
+    if (device < kFastDevices) g_fast[device].store(st, std::memory_order_release);
   }
   cudaSetDevice(prev);
   return LIFT_OK;
@@ -187,7 +194,29 @@ std::vector<Variant>& registry(int op) {
   return g_ops[op];
 }
 
+// The grid of a kernel on a device is a fact of the hardware, so a thread may
+// keep what it has looked up (g_known); the shared map below is for the first
+// time.
+static int64_t persistent_grid_shared(const void* kernel, int threads, size_t smem, int cluster);
+
 int64_t persistent_grid(const void* kernel, int threads, size_t smem, int cluster) {
+  struct Known {
+    int dev;
+    const void* kernel;
+    int64_t grid;
+  };
+  constexpr unsigned kKnown = 64;
+  static thread_local Known known[kKnown] = {};
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  Known& k = known[(reinterpret_cast<uintptr_t>(kernel) >> 4) % kKnown];
+  if (k.kernel == kernel && k.dev == dev && current_state()) return k.grid;
+  const int64_t g = persistent_grid_shared(kernel, threads, smem, cluster);
+  if (g > 0) k = Known{dev, kernel, g};
+  return g;
+}
+
+static int64_t persistent_grid_shared(const void* kernel, int threads, size_t smem, int cluster) {
   static std::mutex mu;
   static std::map<std::pair<int, const void*>, int64_t> cache;
   int dev = -1;
@@ -413,10 +442,20 @@ static int fixed_gemv_t(const Args& a) {
   return id[N <= 256 ? kStagedNarrow : N < 4096 ? kStagedMid : kStaged];
 }
 
+// The op's one default, looked up by name once.
+static int fixed_default(int op) {
+  static const std::vector<int> id = [] {
+    std::vector<int> v;
+    for (int o = 0; o < LIFT_NUM_OPS; ++o) v.push_back(find_variant(o, kDefaultName[o]));
+    return v;
+  }();
+  return id[op];
+}
+
 static int fixed_pick(int op, const Args& a) {
   if (op == LIFT_OP_GEMV) return fixed_gemv(a);
   if (op == LIFT_OP_GEMV_T) return fixed_gemv_t(a);
-  return find_variant(op, kDefaultName[op]);
+  return fixed_default(op);
 }
 
 // The learned ranking: (predicted log-time, variant) of every variant that
@@ -730,7 +769,7 @@ static int pick_variant(int op, const Args& a, cudaStream_t s = nullptr, bool ma
     }
   }
   if (g_policy == LIFT_POLICY_TABLE) v = table_pick(op, a);
-  if (v < 0) v = by_shape ? fixed_pick(op, a) : find_variant(op, kDefaultName[op]);
+  if (v < 0) v = by_shape ? fixed_pick(op, a) : fixed_default(op);
   return v;
 }
 
@@ -866,6 +905,7 @@ lift_status lift_finalize(void) {
   std::lock_guard<std::mutex> lk(g_mu);
   int prev = -1;
   cudaGetDevice(&prev);
+  for (auto& f : g_fast) f.store(nullptr, std::memory_order_release);
   for (auto& kv : g_states) {
     cudaSetDevice(kv.first);
     cudaDeviceSynchronize();

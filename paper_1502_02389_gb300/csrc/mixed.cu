@@ -318,16 +318,15 @@ struct Mixed {
     return (nb + per - 1) / per;
   }
   static lift_status launch(const Variant& v, const Args& a, cudaStream_t s) {
-    DeviceState* st = current_state();
     const int64_t g = grid(v, a);
     if (g <= 0) return set_error(LIFT_ERR_CUDA, std::string("no resident CTA for ") + v.info.name);
-    if (g > st->ws.capacity) return set_error(LIFT_ERR_UNSUPPORTED, "grid exceeds workspace");
+    if (g > a.ws->capacity) return set_error(LIFT_ERR_UNSUPPORTED, "grid exceeds workspace");
     const void* x = a.x;
     const void* y = a.y;
     const float* xs = a.xscale;
     const float* ys = a.yscale;
     int64_t n = a.n;
-    if (g > st->ws.capacity64) return set_error(LIFT_ERR_UNSUPPORTED, "grid exceeds workspace");
+    if (g > a.ws->capacity64) return set_error(LIFT_ERR_UNSUPPORTED, "grid exceeds workspace");
     double* partials = a.ws->partials64;
     unsigned* ticket = a.ws->tickets + 1;
     float* result = a.result;

@@ -371,10 +371,9 @@ struct ReduceF32 {
   }
 
   static lift_status launch(const Variant& v, const Args& a, cudaStream_t s) {
-    DeviceState* st = current_state();
     const int64_t g = grid(v, a);
     if (g <= 0) return set_error(LIFT_ERR_CUDA, std::string("no resident CTA for ") + v.info.name);
-    if (g > st->ws.capacity)
+    if (g > a.ws->capacity)
       return set_error(LIFT_ERR_UNSUPPORTED, "grid exceeds the partials workspace");
     const float* x = static_cast<const float*>(a.x);
     const float* y = static_cast<const float*>(a.y);
@@ -383,7 +382,7 @@ struct ReduceF32 {
     unsigned* ticket = a.ws->tickets;
     float* result = a.result;
     double* result64 = a.result64;
-    int* status = st->ws.status;
+    int* status = a.ws->status;
     uint32_t polls = wait_polls();
     void* args[] = {&x, &y, &n, &partials, &ticket, &result, &result64, &status, &polls};
     lift_status rc =

@@ -184,7 +184,7 @@ struct Scal {
     float alpha = a.alpha;
     const float* x = static_cast<const float*>(a.x);
     float* y = a.out;
-    int* status = current_state()->ws.status;
+    int* status = a.ws->status;
     if constexpr (STAGES == 0) {
       void* args[] = {&n, &alpha, &x, &y};
       if (n <= kAheadTiles * TILE) {

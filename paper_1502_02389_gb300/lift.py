@@ -160,10 +160,29 @@ def _ptr(t) -> Optional[int]:
     return t.data_ptr()
 
 
+def _current_stream_lookup():
+    """A function that returns the current stream's handle.  torch's raw
+    accessors replace ``torch.cuda.current_stream()``, which makes a Stream
+    object, once torch has initialised CUDA: a scal of 2^20 floats submitted
+    from Python took 6.5 us with it and takes 3.2 (the lookups saved in the
+    library included)."""
+    import torch
+    torch.cuda.current_stream()          # initialises CUDA, or raises as it always did
+    get, dev = (getattr(torch._C, n, None) for n in ("_cuda_getCurrentRawStream", "_cuda_getDevice"))
+    if get is None or dev is None:
+        return lambda: torch.cuda.current_stream().cuda_stream
+    return lambda: get(dev())
+
+
+_current_stream = None
+
+
 def _stream(s) -> Optional[int]:
     if s is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        global _current_stream
+        if _current_stream is None:
+            _current_stream = _current_stream_lookup()
+        return _current_stream()
     if isinstance(s, int):
         return s
     return s.cuda_stream
