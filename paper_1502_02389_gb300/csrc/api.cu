@@ -452,7 +452,38 @@ static int fixed_default(int op) {
   return id[op];
 }
 
-static int fixed_pick(int op, const Args& a) {
+static bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+    cudaGetLastError();
+    return true;       // unknown: do not time
+  }
+  return st != cudaStreamCaptureStatusNone;
+}
+
+// Reductions of up to 2^20 elements that the host submits one at a time: one
+// launch, whose last CTA combines, instead of two.  The second launch costs
+// the host 1.6 us, more than it saves on the device (asum, n = 2^20, us per
+// host call: 4.9 with two launches, 4.1 with one; n = 2^10: 4.8, 3.3; n = 2^21:
+// 4.9, 5.0).  In a graph there is no submission and two launches lead (n =
+// 2^20: 3.5 against 4.6).  Same tiles, same partials, same combine: the same
+// bits either way.
+static int one_launch(int op) {
+  static const int ops[] = {LIFT_OP_ASUM, LIFT_OP_DOT, LIFT_OP_NRM2, LIFT_OP_SUM};
+  static const char* const names[] = {"asum_t4096_v4_ldg_p1", "dot_t4096_v4_ldg_p1",
+                                      "nrm2_t4096_v4_ldg_p1", "sum_t4096_v4_ldg_p1"};
+  static const std::vector<int> id = [] {
+    std::vector<int> v(LIFT_NUM_OPS, -1);
+    for (int i = 0; i < 4; ++i) v[ops[i]] = find_variant(ops[i], names[i]);
+    return v;
+  }();
+  return id[op];
+}
+constexpr int64_t kOneLaunchMax = 1 << 20;
+
+// call: the pick is for a call on stream s (lift_pick asks without one)
+static int fixed_pick(int op, const Args& a, cudaStream_t s = nullptr, bool call = false) {
+  if (call && a.n <= kOneLaunchMax && one_launch(op) >= 0 && !capturing(s)) return one_launch(op);
   if (op == LIFT_OP_GEMV) return fixed_gemv(a);
   if (op == LIFT_OP_GEMV_T) return fixed_gemv_t(a);
   return fixed_default(op);
@@ -609,15 +640,6 @@ static double l2_bytes() {
   return (double)l2;
 }
 
-static bool capturing(cudaStream_t s) {
-  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
-    cudaGetLastError();
-    return true;       // unknown: do not time
-  }
-  return st != cudaStreamCaptureStatusNone;
-}
-
 // Time the candidates; returns the fastest, or -1 on any error.
 static int tune_candidates(int op, const Args& a0, const std::vector<int>& cand, cudaStream_t s) {
   DeviceState* st = current_state();
@@ -769,7 +791,7 @@ static int pick_variant(int op, const Args& a, cudaStream_t s = nullptr, bool ma
     }
   }
   if (g_policy == LIFT_POLICY_TABLE) v = table_pick(op, a);
-  if (v < 0) v = by_shape ? fixed_pick(op, a) : fixed_default(op);
+  if (v < 0) v = by_shape ? fixed_pick(op, a, s, may_tune) : fixed_default(op);
   return v;
 }
 
