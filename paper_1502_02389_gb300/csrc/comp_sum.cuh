@@ -62,5 +62,71 @@ __device__ __forceinline__ Comp block_comp(Comp v) {
   return v;
 }
 
+// The end of a reduction whose CTAs leave one FP64 partial each.  One pass (a
+// ticket): the last CTA to arrive adds them.  Two passes (no ticket): a second
+// kernel, launched as a programmatic dependent, adds them in the same order --
+// the same bits -- while the next call is already being scheduled; a last CTA
+// that does so competes with the next call's first loads.  `value` is valid in
+// thread 0.
+template <int THREADS, bool ROOT = false>
+__device__ __forceinline__ void finish64(double value, double* __restrict__ partials, unsigned* ticket,
+                                         float* result, double* result64) {
+  __shared__ bool is_last;
+  __shared__ double red64[kWarp];
+  const int t = threadIdx.x;
+  const int64_t G = gridDim.x;
+  if (ticket == nullptr) {
+    if (t == 0) partials[blockIdx.x] = value;
+    return;
+  }
+  if (t == 0) {
+    partials[blockIdx.x] = value;
+    __threadfence();
+    is_last = atomicAdd(ticket, 1u) == static_cast<unsigned>(G - 1);
+  }
+  __syncthreads();
+  if (!is_last) return;
+  __threadfence();
+  double s = 0.0;
+  for (int64_t i = t; i < G; i += THREADS) s = __dadd_rn(s, __ldcg(partials + i));
+  s = block_tree64<THREADS>(s, red64);
+  if (t == 0) {
+    if (ROOT) s = __dsqrt_rn(s);
+    *result = static_cast<float>(s);
+    if (result64) *result64 = s;
+    *ticket = 0u;
+  }
+}
+
+template <int THREADS, bool ROOT>
+__global__ void __launch_bounds__(THREADS)
+    combine64_kernel(const double* __restrict__ partials, int64_t G, float* result, double* result64) {
+  pdl_trigger();   // the next call's first kernel may be scheduled (it waits for this one)
+  pdl_wait();      // the first pass has finished
+  __shared__ double red64[kWarp];
+  double s = 0.0;
+  for (int64_t i = threadIdx.x; i < G; i += THREADS) s = __dadd_rn(s, __ldcg(partials + i));
+  s = block_tree64<THREADS>(s, red64);
+  if (threadIdx.x == 0) {
+    if (ROOT) s = __dsqrt_rn(s);
+    *result = static_cast<float>(s);
+    if (result64) *result64 = s;
+  }
+}
+
+// Two passes pay from about this many bytes read on: the host submits the
+// second launch while the first kernel runs.
+constexpr int64_t kTwoPassBytes = 16 << 20;
+
+template <int THREADS, bool ROOT = false>
+struct Combine64 {
+  static const void* kernel() { return reinterpret_cast<const void*>(&combine64_kernel<THREADS, ROOT>); }
+  static lift_status launch(const double* partials, int64_t G, float* result, double* result64,
+                            cudaStream_t s) {
+    void* args[] = {&partials, &G, &result, &result64};
+    return launch_config(kernel(), dim3(1), dim3(THREADS), 0, 1, s, args, true);
+  }
+};
+
 }  // namespace
 }  // namespace lift

@@ -84,24 +84,7 @@ __global__ void __launch_bounds__(THREADS)
 #pragma unroll
   for (int l = 1; l < VW; ++l) c = comp_merge(c, acc[l]);
   c = block_comp<THREADS>(c);
-  __shared__ bool is_last;
-  __shared__ double red64[kWarp];
-  if (t == 0) {
-    partials[blockIdx.x] = comp_value(c);
-    __threadfence();
-    is_last = atomicAdd(ticket, 1u) == static_cast<unsigned>(G - 1);
-  }
-  __syncthreads();
-  if (!is_last) return;
-  __threadfence();
-  double s = 0.0;
-  for (int64_t i = t; i < G; i += THREADS) s = __dadd_rn(s, __ldcg(partials + i));
-  s = block_tree64<THREADS>(s, red64);
-  if (t == 0) {
-    *result = static_cast<float>(s);
-    if (result64) *result64 = s;
-    *ticket = 0u;
-  }
+  finish64<THREADS>(comp_value(c), partials, ticket, result, result64);
 }
 
 constexpr int kCompTicket = 2;    // workspace counter of this family
@@ -128,11 +111,14 @@ struct CompReduce {
     int64_t n = a.n;
     if (g > a.ws->capacity64) return set_error(LIFT_ERR_UNSUPPORTED, "grid exceeds workspace");
     double* partials = a.ws->partials64;
-    unsigned* ticket = a.ws->tickets + kCompTicket;
+    const bool two = (OP == LIFT_OP_DOT ? 8 : 4) * n >= kTwoPassBytes;
+    unsigned* ticket = two ? nullptr : a.ws->tickets + kCompTicket;
     float* result = a.result;
     double* result64 = a.result64;
     void* args[] = {&x, &y, &n, &partials, &ticket, &result, &result64};
-    return launch_config(kernel(), dim3((unsigned)g), dim3(THREADS), 0, 1, s, args, true);
+    const lift_status rc =
+        launch_config(kernel(), dim3((unsigned)g), dim3(THREADS), 0, 1, s, args, true);
+    return rc != LIFT_OK || !two ? rc : Combine64<THREADS>::launch(partials, g, result, result64, s);
   }
 };
 

@@ -283,6 +283,13 @@ __global__ void __launch_bounds__(THREADS)
 
   pdl_trigger();   // streaming done: the next call's first kernel may be scheduled
   const Comp c = block_comp<THREADS>(acc);
+  // asum: two passes in long calls (see finish64).  The dots keep their last
+  // CTA: their loops hold 48 to 64 registers, and every form of the end that
+  // was tried moved them to other counts and lost 1 to 8 % (n = 2^28).
+  if constexpr (OP == LIFT_OP_ASUM) {
+    finish64<THREADS>(comp_value(c), partials, ticket, result, result64);
+    return;
+  }
   __shared__ bool is_last;
   __shared__ double red64[kWarp];
   if (t == 0) {
@@ -328,11 +335,14 @@ struct Mixed {
     int64_t n = a.n;
     if (g > a.ws->capacity64) return set_error(LIFT_ERR_UNSUPPORTED, "grid exceeds workspace");
     double* partials = a.ws->partials64;
-    unsigned* ticket = a.ws->tickets + 1;
+    const bool two = OP == LIFT_OP_ASUM && (DT == DT_FP8 ? 1 : 2) * n >= kTwoPassBytes;
+    unsigned* ticket = two ? nullptr : a.ws->tickets + 1;
     float* result = a.result;
     double* result64 = a.result64;
     void* args[] = {&x, &xs, &y, &ys, &n, &partials, &ticket, &result, &result64};
-    return launch_config(kernel(), dim3((unsigned)g), dim3(THREADS), 0, 1, s, args, true);
+    const lift_status rc =
+        launch_config(kernel(), dim3((unsigned)g), dim3(THREADS), 0, 1, s, args, true);
+    return rc != LIFT_OK || !two ? rc : Combine64<THREADS>::launch(partials, g, result, result64, s);
   }
 };
 

@@ -138,8 +138,6 @@ __global__ void __launch_bounds__(kUnThreads)
                      double* result64) {
   constexpr int J = kUnVecs;
   __shared__ float red[kWarp];
-  __shared__ double red64[kWarp];
-  __shared__ bool is_last;
   const int t = threadIdx.x, lane = t & (kWarp - 1);
   const int64_t G = gridDim.x, T = (hi + kUnTile - 1) / kUnTile;
   if (t < 2 && whole_tile(blockIdx.x + t * G, kUnTile, lo, hi, d)) {    // the CTA's first two tiles
@@ -190,24 +188,7 @@ __global__ void __launch_bounds__(kUnThreads)
     }
   }
   pdl_trigger();   // streaming done: the next call's first kernel may be scheduled
-  const double r = f.cta_value(red);
-  if (t == 0) {
-    partials[blockIdx.x] = r;
-    __threadfence();
-    is_last = atomicAdd(ticket, 1u) == static_cast<unsigned>(G - 1);
-  }
-  __syncthreads();
-  if (!is_last) return;
-  __threadfence();
-  double s = 0.0;
-  for (int64_t i = t; i < G; i += kUnThreads) s = __dadd_rn(s, __ldcg(partials + i));
-  s = block_tree64<kUnThreads>(s, red64);
-  if (t == 0) {
-    if (ROOT) s = __dsqrt_rn(s);
-    *result = static_cast<float>(s);
-    if (result64) *result64 = s;
-    *ticket = 0u;
-  }
+  finish64<kUnThreads, ROOT>(f.cta_value(red), partials, ticket, result, result64);
 }
 
 constexpr int kMapVecs = 2, kMapTile = kUnThreads * 4 * kMapVecs;
@@ -286,11 +267,15 @@ struct UnalignedReduce {
     const int64_t per = (T + g - 1) / g;
     g = (T + per - 1) / per;
     double* partials = a.ws->partials64;
-    unsigned* ticket = a.ws->tickets + kUnTicket;
+    const bool two = (F::kTwo ? 8 : 4) * a.n >= kTwoPassBytes;
+    unsigned* ticket = two ? nullptr : a.ws->tickets + kUnTicket;
     float* result = a.result;
     double* result64 = a.result64;
     void* args[] = {&x, &y, &lo, &hi, &d, &partials, &ticket, &result, &result64};
-    return launch_config(kernel(), dim3((unsigned)g), dim3(kUnThreads), 0, 1, s, args, true);
+    const lift_status rc =
+        launch_config(kernel(), dim3((unsigned)g), dim3(kUnThreads), 0, 1, s, args, true);
+    return rc != LIFT_OK || !two ? rc
+                                 : Combine64<kUnThreads, ROOT>::launch(partials, g, result, result64, s);
   }
 };
 
