@@ -10,10 +10,12 @@
 // arguments.  A training step of 2308 shapes and 265 outputs (forward, loss,
 // backward, Adam; host calls included) took 615 us as thirteen launches of
 // one GEMM or reduction each, most of it in the one-CTA loss and in
-// reductions over the 2308 rows by 3 to 18 CTAs; 49 us as five (forward 7.8,
-// loss 7.9, gradients 21.6, Adam 2.2 each alone in a graph).  Bound by
+// reductions over the 2308 rows by 3 to 18 CTAs; 43 us as five (forward 7.6,
+// loss 7.9, gradients 20.2, Adam 1.8 each alone in a graph).  Bound by
 // latency: each launch is one or two dependent phases of copies and
-// shared-memory folds on all SMs.  Other sizes run the one-operation kernels.
+// shared-memory folds on all SMs, and each is a programmatic dependent of the
+// one before it (49 us as plain launches).  Other sizes run the one-operation
+// kernels.
 //
 // The model predicts one log-time per kernel variant from the features of a
 // call; the autotuner's measurements are its training data (the paper's
@@ -112,6 +114,8 @@ __global__ void __launch_bounds__(kLossThreads)
                int64_t count, float inv, float* __restrict__ dP, float* __restrict__ loss) {
   __shared__ float red[kWarp];
   __shared__ float part;
+  pdl_trigger();   // the next launch may be scheduled (it waits for this one)
+  pdl_wait();      // the launch before has finished
   cg::cluster_group cl = cg::this_cluster();
   const int64_t t = (int64_t)blockIdx.x * kLossThreads + threadIdx.x;
   const int64_t kAll = (int64_t)gridDim.x * kLossThreads;
@@ -166,6 +170,8 @@ __device__ __forceinline__ void cp4(float* dst, const float* src) {
 __device__ __forceinline__ void cp16(float* dst, const float* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
 }
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void cp_wait_all_but_one() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
 __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // n floats, by the whole CTA; vec: both sides 16-byte aligned
@@ -233,6 +239,8 @@ __global__ void __launch_bounds__(512)
   float* xs = h2;
   const int r0 = blockIdx.x * kRows, rows = B - r0 < kRows ? B - r0 : kRows;
   const bool vec = reinterpret_cast<uintptr_t>(W1) % 16 == 0;   // so are the other matrices
+  // (no early trigger: the next launch's CTAs beside these took 3 us from them)
+  pdl_wait();      // the launch before has finished
   for (int i = threadIdx.x; i < kRows * d; i += blockDim.x) {
     const int r = i / d, k = i % d;
     if (r < rows) cp4(xs + k * kPitch + r, X + (size_t)r0 * d + i);
@@ -240,11 +248,15 @@ __global__ void __launch_bounds__(512)
   }
   cp_flat(w1, W1, d * kH, vec);
   cp_flat(w2, W2, kH * kH, vec);
+  cp_commit();
   if (CW == V) cp_flat(w3, W3, kH * V, vec);
-  cp_wait();
+  cp_commit();
+  cp_wait_all_but_one();
   __syncthreads();
   hidden_layer(d, xs, w1, b1, r0, rows, Z1, H1, h1);
   hidden_layer(kH, h1, w2, b2, r0, rows, Z2, H2, h2);
+  cp_wait();
+  __syncthreads();
   for (int c0 = 0; c0 < V; c0 += CW) {
     const int cw = V - c0 < CW ? V - c0 : CW;
     if (CW != V) {
@@ -277,34 +289,47 @@ __global__ void __launch_bounds__(512)
 // dZ2 = (dP W3^T) * [Z2 > 0] and dZ1 = (dZ2 W2^T) * [Z1 > 0] of kRows rows
 // per CTA.  W3 (in chunks of CW output columns) and W2 are staged in shared
 // memory with an odd pitch, so that 32 threads that walk 32 rows of W
-// together read 32 banks; the sum over a row's columns is split between two
-// halves of the CTA.
+// together read 32 banks; the sum over a row's columns is split between four
+// quarters of the CTA.
 constexpr int kActThreads = 512;
 
+// Thread (units j and j + 32, rows 4g .. 4g+3, a quarter of the columns): one
+// broadcast read of four rows serves two units.
 __device__ __forceinline__ void back_layer(int cw, int pitch, const float* W, const float* in,
-                                           float (&acc)[4]) {
-  // thread (unit j, rows 4g .. 4g+3, half of the columns)
-  const int j = threadIdx.x % kH, g = threadIdx.x / kH % (kRows / 4), half = threadIdx.x / 256;
-  const int c0 = half * (cw / 2), c1 = half ? cw : cw / 2;
+                                           float (&acc)[2][4]) {
+  const int j = threadIdx.x % kWarp, g = threadIdx.x / kWarp % (kRows / 4), part = threadIdx.x / 128;
+  const int c0 = cw * part / 4, c1 = cw * (part + 1) / 4;
 #pragma unroll 8
-  for (int c = c0; c < c1; ++c) fma4(acc, W[j * pitch + c], in + c * kPitch + 4 * g);
+  for (int c = c0; c < c1; ++c) {
+    fma4(acc[0], W[j * pitch + c], in + c * kPitch + 4 * g);
+    fma4(acc[1], W[(j + kWarp) * pitch + c], in + c * kPitch + 4 * g);
+  }
 }
 
-// adds the halves, applies the gate, leaves the result in `out` and in global memory
-__device__ __forceinline__ void gate_layer(const float (&acc)[4], float* halves, const float* gate,
+// adds the quarters, applies the gate, leaves the result in `out` and in global memory
+__device__ __forceinline__ void gate_layer(const float (&acc)[2][4], float* parts, const float* gate,
                                            int r0, int rows, float* out, float* __restrict__ D) {
-  const int j = threadIdx.x % kH, g = threadIdx.x / kH % (kRows / 4);
-  if (threadIdx.x >= 256)
-    *reinterpret_cast<float4*>(halves + j * kPitch + 4 * g) = make_float4(acc[0], acc[1], acc[2], acc[3]);
-  __syncthreads();
-  if (threadIdx.x < 256) {
+  const int j = threadIdx.x % kWarp, g = threadIdx.x / kWarp % (kRows / 4), part = threadIdx.x / 128;
+  if (part > 0) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int r = 4 * g + q;
-      const float v = gate[j * kPitch + r] > 0.f ? acc[q] + halves[j * kPitch + r] : 0.f;
-      out[j * kPitch + r] = v;
-      if (r < rows) D[(size_t)(r0 + r) * kH + j] = v;
-    }
+    for (int h = 0; h < 2; ++h)
+      *reinterpret_cast<float4*>(parts + ((part - 1) * kH + j + kWarp * h) * kPitch + 4 * g) =
+          make_float4(acc[h][0], acc[h][1], acc[h][2], acc[h][3]);
+  }
+  __syncthreads();
+  if (part == 0) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int r = 4 * g + q, u = j + kWarp * h;
+        float v = acc[h][q];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) v += parts[(k * kH + u) * kPitch + r];
+        v = gate[u * kPitch + r] > 0.f ? v : 0.f;
+        out[u * kPitch + r] = v;
+        if (r < rows) D[(size_t)(r0 + r) * kH + u] = v;
+      }
   }
   __syncthreads();
 }
@@ -319,10 +344,12 @@ __global__ void __launch_bounds__(kActThreads)
   float* h1 = dps + CW * kPitch;                    // [kH][kPitch]
   float* h2 = h1 + kH * kPitch;
   float* d0 = h2 + kH * kPitch;
-  float* halves = d0 + kH * kPitch;
-  float* w2 = halves + kH * kPitch;                 // [kH][kH + 1]
+  float* parts = d0 + kH * kPitch;                  // [3][kH][kPitch]
+  float* w2 = parts + 3 * kH * kPitch;              // [kH][kH + 1]
   float* w3 = w2 + kH * (kH + 1);                   // [kH][pitch]
   const int t = threadIdx.x, r0 = blockIdx.x * kRows, rows = B - r0 < kRows ? B - r0 : kRows;
+  pdl_trigger();   // the next launch may be scheduled (it waits for this one)
+  pdl_wait();      // the launch before has finished
   for (int i = t; i < kRows * kH; i += kActThreads) {    // relu(Z) > 0 where Z > 0
     const int r = i / kH, j = i % kH;
     if (r < rows) {
@@ -333,7 +360,7 @@ __global__ void __launch_bounds__(kActThreads)
     }
   }
   for (int i = t; i < kH * kH; i += kActThreads) cp4(w2 + i / kH * (kH + 1) + i % kH, W2 + i);
-  float acc[4] = {0.f, 0.f, 0.f, 0.f};
+  float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
   const int warp = t / kWarp, lane = t % kWarp;
   for (int c0 = 0; c0 < V; c0 += CW) {
     const int cw = V - c0 < CW ? V - c0 : CW;
@@ -349,20 +376,21 @@ __global__ void __launch_bounds__(kActThreads)
     back_layer(cw, pitch, w3, dps, acc);
     __syncthreads();                                // the chunk is read before the next one lands
   }
-  gate_layer(acc, halves, h2, r0, rows, d0, D0);
-  float acc1[4] = {0.f, 0.f, 0.f, 0.f};
+  gate_layer(acc, parts, h2, r0, rows, d0, D0);
+  float acc1[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
   back_layer(kH, kH + 1, w2, d0, acc1);             // dZ1_i = sum_j dZ2_j W2[i][j]
-  gate_layer(acc1, halves, h1, r0, rows, h2, D1);   // (h2 is no longer read)
+  gate_layer(acc1, parts, h1, r0, rows, h2, D1);    // (h2 is no longer read)
 }
 
 // Weight and bias gradients: out[i][c] = sum_r L[r][i] R[r][c] and, for the
 // biases, sum_r R[r][c], for the pairs (H2, dP), (H1, dZ2) and (X, dZ1).  A
 // cluster of kGradCtas CTAs takes 32 columns c and every i <= 64, each CTA a
 // contiguous part of the rows: copied to shared memory up to kGradRows at a
-// time with every copy in flight at once (2308 x 265: 21.6 us for both
-// gradient launches, 34.4 when the rows were read from global memory as they
-// were folded, waiting on loads), folded in kGradShares shares by thread (share, 8 consecutive i, c),
-// and the shares added in order through distributed shared memory.
+// time in two halves, the second in flight while the first is folded (2308 x
+// 265: 20.2 us for both gradient launches, 34.4 when the rows were read from
+// global memory as they were folded, waiting on loads), folded in kGradShares
+// shares by thread (share, 8 consecutive i, c), and the shares added in order
+// through distributed shared memory.
 constexpr int kGradCtas = 8, kGradI = 8, kGradGroups = kH / kGradI, kGradShares = 4;
 constexpr int kGradThreads = kGradShares * kGradGroups * kWarp, kGradRows = 304;
 
@@ -394,6 +422,8 @@ __global__ void __launch_bounds__(kGradThreads)
   float acc[kGradI], bs = 0.f;
 #pragma unroll
   for (int q = 0; q < kGradI; ++q) acc[q] = 0.f;
+  pdl_trigger();   // the next launch may be scheduled (it waits for this one)
+  pdl_wait();      // the launch before has finished
   if (li < kH)                                           // columns past L stay zero
     for (int e = threadIdx.x; e < kGradRows * kH; e += kGradThreads)
       if (e % kH >= li) ls[e] = 0.f;
@@ -401,21 +431,32 @@ __global__ void __launch_bounds__(kGradThreads)
     const int rows = b1 - r0 < kGradRows ? b1 - r0 : kGradRows;
     const float* L = job.L + (size_t)r0 * li;
     const float* R = job.R + (size_t)r0 * rc + c0;
-    if (job.vec) {
-      const int l4 = li / 4;
-      for (int e = threadIdx.x; e < rows * l4; e += kGradThreads)
-        cp16(ls + e / l4 * kH + e % l4 * 4, L + 4 * (size_t)e);
-    } else {
-      for (int e = threadIdx.x; e < rows * li; e += kGradThreads) cp4(ls + e / li * kH + e % li, L + e);
+    const int mid = rows / 2;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {                        // the second half lands while the first is folded
+      const int q0 = h ? mid : 0, q1 = h ? rows : mid;
+      if (job.vec) {
+        const int l4 = li / 4;
+        for (int e = q0 * l4 + threadIdx.x; e < q1 * l4; e += kGradThreads)
+          cp16(ls + e / l4 * kH + e % l4 * 4, L + 4 * (size_t)e);
+      } else {
+        for (int e = q0 * li + threadIdx.x; e < q1 * li; e += kGradThreads)
+          cp4(ls + e / li * kH + e % li, L + e);
+      }
+      for (int r = q0 + threadIdx.x / kWarp; r < q1; r += kGradThreads / kWarp) {
+        if (c0 + lane < rc) cp4(rs + r * kWarp + lane, R + (size_t)r * rc + lane);
+        else rs[r * kWarp + lane] = 0.f;
+      }
+      cp_commit();
     }
-    for (int r = threadIdx.x / kWarp; r < rows; r += kGradThreads / kWarp) {
-      if (c0 + lane < rc) cp4(rs + r * kWarp + lane, R + (size_t)r * rc + lane);
-      else rs[r * kWarp + lane] = 0.f;
-    }
-    cp_wait();
-    __syncthreads();
-    if (i0 < li || grp == 0) {
-      const int ra = rows * share / kGradShares, rb = rows * (share + 1) / kGradShares;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      if (h == 0) cp_wait_all_but_one();
+      else cp_wait();
+      __syncthreads();
+      if (i0 >= li && grp != 0) continue;
+      const int q0 = h ? mid : 0, half = h ? rows - mid : mid;
+      const int ra = q0 + half * share / kGradShares, rb = q0 + half * (share + 1) / kGradShares;
 #pragma unroll 4
       for (int r = ra; r < rb; ++r) {
         const float v = rs[r * kWarp + lane];
@@ -464,6 +505,8 @@ __global__ void __launch_bounds__(kGradThreads)
 __global__ void adam(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
                      float* __restrict__ v, int64_t count, float lr, float b1, float b2, float eps,
                      float c1, float c2) {
+  pdl_trigger();   // the next launch may be scheduled (it waits for this one)
+  pdl_wait();      // the launch before has finished
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < count;
        i += (int64_t)gridDim.x * blockDim.x) {
     const float gi = g[i];
@@ -528,7 +571,7 @@ bool fused_shape(int d, int h1, int h2) { return h1 == kH && h2 == kH && d <= kH
 
 lift_status forward_fused(int d, int V, const float* p, const Layout& L, const float* X, int B,
                           float* Z1, float* H1, float* Z2, float* H2, float* P, cudaStream_t s) {
-  const int CW = V < kFwdColumns ? V : kFwdColumns;
+  int CW = V < kFwdColumns ? V : kFwdColumns;
   int threads = (CW + kWarp - 1) / kWarp * kWarp;    // one output column per thread if it can be
   threads = threads < 256 ? 256 : threads > 512 ? 512 : threads;
   const size_t smem = sizeof(float) * ((size_t)kH * CW + 2 * kH * kH + 2 * kH * kPitch);
@@ -536,9 +579,11 @@ lift_status forward_fused(int d, int V, const float* p, const Layout& L, const f
       cudaFuncSetAttribute(mlp_forward_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, 208 * 1024),
       "mlp_forward shared memory");
   if (rc != LIFT_OK) return rc;
-  mlp_forward_fused<<<(B + kRows - 1) / kRows, threads, smem, s>>>(
-      B, d, V, CW, p + L.W1, p + L.b1, p + L.W2, p + L.b2, p + L.W3, p + L.b3, X, Z1, H1, Z2, H2, P);
-  return cuda_check(cudaGetLastError(), "mlp_forward launch");
+  const float *W1 = p + L.W1, *b1 = p + L.b1, *W2 = p + L.W2, *b2 = p + L.b2, *W3 = p + L.W3,
+              *b3 = p + L.b3;
+  void* args[] = {&B, &d, &V, &CW, &W1, &b1, &W2, &b2, &W3, &b3, &X, &Z1, &H1, &Z2, &H2, &P};
+  return launch_config(reinterpret_cast<const void*>(&mlp_forward_fused), dim3((B + kRows - 1) / kRows),
+                       dim3(threads), smem, 1, s, args, true);
 }
 
 lift_status backward_fused(int d, int V, const float* p, const Layout& L, const float* X, int B,
@@ -546,15 +591,16 @@ lift_status backward_fused(int d, int V, const float* p, const Layout& L, const 
                            float* grads, cudaStream_t s) {
   constexpr int kChunk = 288;                        // output columns staged at a time, at most
   const int chunks = (V + kChunk - 1) / kChunk, CW = (V + chunks - 1) / chunks;
-  const size_t smem = sizeof(float) * ((size_t)CW * kPitch + 4 * kH * kPitch + kH * (kH + 1) +
+  const size_t smem = sizeof(float) * ((size_t)CW * kPitch + 6 * kH * kPitch + kH * (kH + 1) +
                                        (size_t)kH * (CW | 1));
   lift_status rc = cuda_check(cudaFuncSetAttribute(mlp_back_rows,
                                                    cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   144 * 1024), "mlp_backward shared memory");
+                                                   152 * 1024), "mlp_backward shared memory");
   if (rc != LIFT_OK) return rc;
-  mlp_back_rows<<<(B + kRows - 1) / kRows, kActThreads, smem, s>>>(B, V, CW, p + L.W2, p + L.W3, H1,
-                                                                  H2, dP, D0, D1);
-  rc = cuda_check(cudaGetLastError(), "mlp_backward launch");
+  const float *W2 = p + L.W2, *W3 = p + L.W3;
+  void* rows_args[] = {&B, &V, const_cast<int*>(&CW), &W2, &W3, &H1, &H2, &dP, &D0, &D1};
+  rc = launch_config(reinterpret_cast<const void*>(&mlp_back_rows), dim3((B + kRows - 1) / kRows),
+                     dim3(kActThreads), smem, 1, s, rows_args, true);
   if (rc != LIFT_OK) return rc;
   const int t3 = (V + kWarp - 1) / kWarp, t64 = kH / kWarp;
   const int hv = aligned(H1, 16) && aligned(H2, 16), xv = aligned(X, 16) && d % 4 == 0;
@@ -568,7 +614,7 @@ lift_status backward_fused(int d, int V, const float* p, const Layout& L, const 
   void* args[] = {&B, &jobs};
   return launch_config(reinterpret_cast<const void*>(&mlp_weight_grads),
                        dim3((unsigned)(t3 + 2 * t64) * kGradCtas), dim3(kGradThreads), kGradSmem,
-                       kGradCtas, s, args);
+                       kGradCtas, s, args, true);
 }
 
 bool bad_shape(int d, int h1, int h2, int V) { return d < 1 || h1 < 1 || h2 < 1 || V < 1; }
@@ -621,7 +667,7 @@ lift_status lift_mlp_loss(const float* P, const float* T, const float* mask, int
   const int ctas = loss_cluster(k);
   void* args[] = {&P, &T, &mask, &count, &inv_measured, &dP, &loss};
   return launch_config(k, dim3(ctas), dim3(kLossThreads), 0, ctas, static_cast<cudaStream_t>(stream),
-                       args);
+                       args, true);
 }
 
 lift_status lift_mlp_backward(int d_in, int h1, int h2, int V, const float* params, const float* X,
@@ -667,9 +713,10 @@ lift_status lift_mlp_adam(float* params, const float* grads, float* m, float* v,
   const float c1 = 1.f - powf(beta1, (float)t), c2 = 1.f - powf(beta2, (float)t);
   int blocks = (int)((count + 255) / 256);
   if (blocks > 1024) blocks = 1024;
-  adam<<<blocks, 256, 0, static_cast<cudaStream_t>(stream)>>>(params, grads, m, v, count, lr, beta1,
-                                                               beta2, eps, c1, c2);
-  return cuda_check(cudaGetLastError(), "mlp_adam launch");
+  void* args[] = {&params, &grads, &m, &v, &count, &lr, &beta1, &beta2, &eps, const_cast<float*>(&c1),
+                  const_cast<float*>(&c2)};
+  return launch_config(reinterpret_cast<const void*>(&adam), dim3(blocks), dim3(256), 0, 1,
+                       static_cast<cudaStream_t>(stream), args, true);
 }
 
 }  // extern "C"
