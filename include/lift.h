@@ -35,7 +35,9 @@
  *    y <- b*y, and with M == 0 does nothing.
  *  - A pointer that is not aligned for a variant's vector width or for
  *    TMA bulk copies (16 B) makes the library use the same variant family's
- *    guarded scalar-load form instead; it is not an error.
+ *    guarded scalar-load form instead; it is not an error.  A vector op
+ *    called without a variant id reads slices that start off a 16-byte
+ *    boundary in 16-byte loads all the same.
  *  - The reductions use a per-device workspace allocated by lift_init
  *    (partials, ticket counters, a status word), one slot per stream for up
  *    to 8 streams of a device; calls on the same stream are ordered by it.
@@ -405,7 +407,8 @@ lift_status lift_dot_ex_v(int variant, lift_dtype t, const void* x, const float*
  * Both learned policies choose only among the variants that run as
  * themselves on the call's arguments (vector loads need the pointers and,
  * for gemv and gemv-T, the row pitch aligned to the vector width); an
- * explicit or FIXED variant that cannot runs its guarded fallback.  Their
+ * explicit variant that cannot runs its guarded fallback, and the FIXED
+ * pick of a vector op its unaligned form.  Their
  * picks are memoised per (op, shape, pointer and pitch alignment), so a
  * repeated call shape costs a table lookup; loading weights clears the
  * memo.
@@ -424,7 +427,9 @@ lift_status lift_set_policy(int policy, const char* path);
 lift_status lift_tune_stats(int64_t* tuned_shapes, int64_t* timed_launches);
 /* Force `variant` for `op` (-1 clears the override). */
 lift_status lift_set_variant(int op, int variant);
-/* The variant the current policy would use for a dense call (aligned
+/* (A reduction of up to 2^20 elements that is called outside stream capture
+ * runs the one-launch form of this variant's tiles: the same bits.)
+ * The variant the current policy would use for a dense call (aligned
  * pointers, lda = N).  M, N: gemv / gemv-T shape (else 0). */
 lift_status lift_pick(int op, int64_t n, int64_t M, int64_t N, int* variant);
 
