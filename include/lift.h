@@ -40,7 +40,9 @@
  *    boundary in 16-byte loads all the same.
  *  - The reductions use a per-device workspace allocated by lift_init
  *    (partials, ticket counters, a status word), one slot per stream for up
- *    to 8 streams of a device; calls on the same stream are ordered by it.
+ *    to 8 streams of a device; calls on the same stream are ordered by it,
+ *    whichever host threads make them (a call submits all its launches
+ *    before another thread's call on that stream submits any).
  *    Calls on more than 8 streams at once share slots and can race (and
  *    after 4096 distinct stream handles the assignment starts afresh).
  *  - Most kernels are launched as programmatic dependents of the kernel
@@ -399,7 +401,8 @@ lift_status lift_dot_ex_v(int variant, lift_dtype t, const void* x, const float*
  *                      allocated and freed around the timing).  The fastest
  *                      is cached per (op, shape, alignment); the first such
  *                      call waits for the timing (one timing runs at a time;
- *                      other threads' picks do not wait for it).  A call made while its
+ *                      other threads' picks do not wait for it, their
+ *                      calls on the same stream do).  A call made while its
  *                      stream is being captured into a CUDA graph,
  *                      lift_pick and the batch never time: they use a
  *                      cached winner or the plain learned pick.  Loading

@@ -124,6 +124,7 @@ static lift_status init_device(int device) {
     if (rc == LIFT_OK)
       rc = cuda_check(cudaMemset(w.tickets, 0, kTicketSlots * sizeof(unsigned)), "memset");
     w.status = status;
+    w.mu = &st->slot_mu[i];
     w.capacity = kPartialCapacity;
     w.capacity64 = kPartial64Capacity;
   }
@@ -840,6 +841,10 @@ static lift_status run(int op, int variant, const Args& a0, void* stream) {
   const cudaStream_t s = static_cast<cudaStream_t>(stream);
   Args a = a0;
   a.ws = stream_workspace(st, s);
+  // A call of two launches leaves partials in the slot between them, and a
+  // timing of candidates uses the slot on a stream of its own: another host
+  // thread's call on this stream comes before or after all of it.
+  std::lock_guard<std::mutex> slot_lk(*a.ws->mu);
   const Variant* v = nullptr;
   lift_status rc = resolve(op, variant, a, &v, s, true);
   if (rc != LIFT_OK) return rc;

@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -26,6 +27,7 @@ struct Workspace {
   double* partials64 = nullptr;    // per-CTA FP64 partials (sum, compensation pairs)
   unsigned* tickets = nullptr;     // one-pass "last CTA" counters (kept at 0 between calls)
   int* status = nullptr;           // device status word (0 = ok, else lift_status), shared
+  std::mutex* mu = nullptr;        // held while a call submits its launches (run, api.cu)
   int64_t capacity = 0;            // fp32 partial slots
   int64_t capacity64 = 0;          // FP64 partial slots
 };
@@ -41,6 +43,7 @@ struct DeviceState {
   int sm_count = 0;
   Workspace ws;                    // slot 0 (also the capacities and the status word)
   Workspace more[kWsSlots - 1];    // slots 1 ..
+  std::mutex slot_mu[kWsSlots];    // the slots' mutexes
 };
 
 DeviceState* current_state();  // state of the current device, or nullptr
