@@ -18,7 +18,7 @@ import math
 
 from .patterns import (AsScalar, AsVector, C, Id, Iterate, Join, Map, MapLocal, MapSeq,
                        MapWorkgroup, PadTo, PartRed, Reduce, ReduceSeq, ReduceSeqComp, Reorder,
-                       ReorderStride, Split, ToGlobal, ToLocal, Vect, Zip, ZipWith, abs_,
+                       ReorderStride, Split, ToGlobal, ToLocal, TreeComp, Vect, Zip, ZipWith, abs_,
                        absAndPlus, add, add64, fold, id_, mul3, mult, mult_by, sqrt64, square,
                        to_f32, to_f64)
 
@@ -232,6 +232,14 @@ def grouped_dot(vw: int, J: int, group: int = GEMV_GROUP):
     return C(ReduceSeqComp(add), Join(), Map(value), Split(group), PadTo(Jp))
 
 
+def partials_combine(P: int):
+    """[P] fp32 partials of one output -> [1]: lane l of a warp takes
+    partials l, l+32, ... with the compensated reduce-seq, and the lanes'
+    (sum, compensation) pairs go through the halving tree (tree-comp)."""
+    per = max(1, math.ceil(P / WARP))
+    return C(TreeComp(), Split(per), ReorderStride(s=WARP), PadTo(WARP * per))
+
+
 def gemv_row_variant(N: int, vw: int, lanes: int = WARP):
     """Expression of one row of the gemv kernel: ``lanes`` threads share the
     row; lane l takes vectors l, l+lanes, ... of the zero-padded row
@@ -259,20 +267,16 @@ def gemv_split_z_variant(M: int, N: int, alpha, vw: int, threads: int, L: int, S
     split into S segments of L elements; a CTA of ``threads`` folds a
     segment (thread t takes vectors t, t+threads, ... in order and folds
     them with ``grouped_dot``, then ``block_tree``); the S segment partials
-    of the row are added by one warp (lane l adds partials l, l+32, ...
-    with the compensated reduce-seq, then a halving tree) and multiplied by
-    alpha -- the partial-reduction rule of Fig. 3 applied to each row's
-    reduce."""
+    of the row go through
+    ``partials_combine`` and the result is multiplied by alpha -- the
+    partial-reduction rule of Fig. 3 applied to each row's reduce."""
     chunk = threads * vw
     assert L % chunk == 0 and S * L >= N
     J = L // chunk
     segment = C(block_tree(threads), Join(), MapLocal(grouped_dot(vw, J)),
                 Split(J), ReorderStride(s=threads), AsVector(vw) if vw > 1 else Id())
-    per = max(1, math.ceil(S / WARP))
-    lanes = C(halving_tree(add), Join(), MapLocal(ReduceSeqComp(add)), Split(per),
-              ReorderStride(s=WARP), PadTo(WARP * per))
-    row = C(Join(), MapWorkgroup(lanes), Split(S), Join(), MapWorkgroup(segment), Split(L),
-            PadTo(S * L), ZipWith("x"))
+    row = C(Join(), MapWorkgroup(partials_combine(S)), Split(S), Join(), MapWorkgroup(segment),
+            Split(L), PadTo(S * L), ZipWith("x"))
     return C(Map(mult_by(alpha)), Join(), Map(row))
 
 
@@ -287,18 +291,15 @@ def gemv_t_z_variant(M: int, N: int, alpha, B: int, RB: int, passes: int = 1,
     with clusters of ``cluster`` blocks: each cluster's consecutive block
     partials added in order, then the cluster sums added in order with the
     compensated reduce-seq (the partial reduction of Fig. 3d applied to the
-    block partials); two pass: lane l of one warp adds partials l, l+32,
-    ..., then a halving tree over the lanes -- and multiplied by alpha."""
+    block partials); two pass: ``partials_combine``, one warp per column --
+    and multiplied by alpha."""
     if passes == 1 and cluster > 1:
         assert RB % cluster == 0
         combine = C(ReduceSeqComp(add), Join(), Map(ReduceSeq(add, 0)), Split(cluster))
     elif passes == 1:
         combine = ReduceSeqComp(add)
     else:
-        per = max(1, math.ceil(RB / WARP))
-        lanes = C(halving_tree(add), Join(), MapLocal(ReduceSeqComp(add)), Split(per),
-                  ReorderStride(s=WARP), PadTo(WARP * per))
-        combine = C(Join(), MapWorkgroup(lanes), Split(RB))     # one warp per column
+        combine = C(Join(), MapWorkgroup(partials_combine(RB)), Split(RB))   # one warp per column
     Bp = math.ceil(B / group) * group
     block = C(ReduceSeqComp(add), Join(), Map(ReduceSeq(fold(add, mult), 0)), Split(group),
               PadTo(Bp))

@@ -205,6 +205,21 @@ def ReduceSeqComp(f=None):
 
 
 @dataclass(frozen=True)
+class TreeComp(Expr):
+    """[T][K] -> [1], T a multiple of 32: map(reduce-seq-comp) over the T
+    rows, whose (sum, compensation) pairs then go through halving trees
+    unrounded -- one over each 32 rows and, with T > 32, one over their T/32
+    results padded with zeros to 32.  A merge of element j with element j + o
+    adds the compensations and then the sums with TwoSum (Knuth), whose
+    rounding error is added to the compensation; the result is s + c (s
+    itself when s is not finite).  In exact arithmetic this is
+    reduce(add, 0) . join."""
+
+    def __repr__(self) -> str:
+        return "tree-comp"
+
+
+@dataclass(frozen=True)
 class Zip(Expr):
     """zip(a, b): consumes a 2-tuple of equal-length arrays (Table 1)."""
 
@@ -451,6 +466,10 @@ def infer(e, t, ctx: Tuple[str, ...] = ()):
             raise PatternTypeError(f"{e.kind} needs a one-dimensional input, got {t.dims}")
         _reduce_fun_check(e.f, t)
         return t.with_dims((1,), pair=False)
+    if isinstance(e, TreeComp):
+        if len(t.dims) != 2 or t.dims[0] % 32 != 0 or t.dims[0] > 1024 or t.pair or t.vw != 1:
+            raise PatternTypeError(f"tree-comp of {t.dims}")
+        return t.with_dims((1,))
     if isinstance(e, Split):
         if e.n < 1 or len(t.dims) < 1 or t.dims[0] % e.n != 0:
             raise PatternTypeError(f"split-{e.n} of an outer dimension {t.dims[:1]}")
@@ -673,6 +692,19 @@ def _comp_fold_axis(v, ax: int):
     ReduceSeqComp), every operation in the mode's arithmetic (numpy float32
     arithmetic rounds each operation to nearest, as the kernels' explicit
     fp32 operations do)."""
+    s, c = _comp_pairs(v, ax)
+    return _comp_value(s, c)
+
+
+def _comp_value(s, c):
+    if s.dtype.kind == "f":
+        with np.errstate(invalid="ignore", over="ignore"):
+            return np.where(np.isfinite(s), s + c, s)
+    return s + c
+
+
+def _comp_pairs(v, ax: int):
+    """The (sum, compensation) accumulators of the fold."""
     if isinstance(v, Pair):
         raise PatternTypeError("compensated reduction over pairs")
     d = np.asarray(v.data)
@@ -688,9 +720,22 @@ def _comp_fold_axis(v, ax: int):
             big = np.abs(s) >= np.abs(t)
             c = c + np.where(big, (s - u) + t, (t - u) + s)
             s = u
-        if d.dtype.kind == "f":
-            return np.where(np.isfinite(s), s + c, s)
-    return s + c
+    return s, c
+
+
+def _comp_tree(s, c, ax: int):
+    """32 pairs along axis ``ax`` through a halving tree (see TreeComp)."""
+    o = s.shape[ax] // 2
+    with np.errstate(invalid="ignore", over="ignore"):
+        while o:
+            lo, hi = (np.take(s, range(k, k + o), axis=ax) for k in (0, o))
+            cc = np.take(c, range(o), axis=ax) + np.take(c, range(o, 2 * o), axis=ax)
+            u = lo + hi
+            bp = u - lo
+            c = cc + ((lo - (u - bp)) + (hi - bp))
+            s = u
+            o //= 2
+    return s, c
 
 
 # ---------------------------------------------------------------------------
@@ -721,6 +766,18 @@ def _eval(e, v, nb: int, ar: _Arith, env: Dict[str, np.ndarray]):
         else:
             acc = _fold_axis(ar, e.f, e.z, v, nb)
         return Arr(np.expand_dims(np.asarray(acc), nb), v.vw)
+    if isinstance(e, TreeComp):
+        s, c = _comp_pairs(v, nb + 1)
+        T = s.shape[nb]
+        if T > 32:
+            def warps(a):
+                return a.reshape(a.shape[:nb] + (T // 32, 32) + a.shape[nb + 1:])
+            s, c = _comp_tree(warps(s), warps(c), nb + 1)
+            pad = [(0, 0)] * s.ndim
+            pad[nb] = (0, 32 - T // 32)
+            s, c = (np.pad(np.take(a, 0, axis=nb + 1), pad[:-1]) for a in (s, c))
+        s, c = _comp_tree(s, c, nb)
+        return Arr(np.asarray(_comp_value(s, c)), v.vw)
     if isinstance(e, Split):
         def sp(d):
             m = d.shape[nb]

@@ -1,5 +1,6 @@
 // Compensated summation helpers shared by the mixed-precision and the
-// compensated fp32 reductions: a (sum, compensation) pair updated with
+// compensated fp32 reductions and by the trees of the split-row gemv and of
+// the combines of row partials: a (sum, compensation) pair updated with
 // Knuth's TwoSum (the rounding error of every add is carried exactly in the
 // compensation), merged pairwise across a warp and a CTA.
 #pragma once
@@ -30,6 +31,9 @@ __device__ __forceinline__ Comp comp_merge(Comp a, const Comp& b) {
 __device__ __forceinline__ double comp_value(const Comp& a) {
   return isfinite(a.s) ? __dadd_rn((double)a.s, (double)a.c) : (double)a.s;
 }
+
+// the pair's value in fp32, rounded once
+__device__ __forceinline__ float comp_value32(const Comp& a) { return neumaier_value(a.s, a.c); }
 
 __device__ __forceinline__ Comp warp_comp(Comp v) {
 #pragma unroll

@@ -4,7 +4,8 @@
 // Per column, the row block's rows are folded in groups of 32 in row order
 // from zero and the group sums added with Neumaier's compensated step; the
 // RB block values are added as the 32 lanes of a warp add them (lane l
-// takes blocks l, l+32, ..., then a halving tree) -- the bits of
+// takes blocks l, l+32, ..., then a halving tree of (sum, compensation)
+// pairs) -- the bits of
 // gemv_t_kernel's and gemv_t_staged's two-pass forms.  A thread here owns Q
 // column vectors THREADS * VW apart, so that
 //  * with VW == 1 a matrix whose rows are not whole 16-byte granules is
@@ -25,7 +26,7 @@
 // (113); 32 x 1000000: 23.5 (144); 1000 x 777: 6.2 (52).  Two columns per
 // thread with every CTA that fits lead four columns on 4 CTAs per SM (8191 x
 // 8191: 54.1) and 64- or 32-thread CTAs (65.5, 59.9).
-#include "lift_internal.cuh"
+#include "comp_sum.cuh"
 
 namespace lift {
 
@@ -135,14 +136,14 @@ __global__ void __launch_bounds__(kColsCombineThreads)
   pdl_wait();      // the first pass has finished
   const int64_t j = (int64_t)blockIdx.x * kColsCombineThreads + threadIdx.x;
   if (j >= N) return;
-  float v[kColsTree];
+  Comp v[kColsTree];
 #pragma unroll
-  for (int b = 0; b < kColsTree; ++b) v[b] = b < RB ? __ldcg(partials + b * N + j) : 0.f;
+  for (int b = 0; b < kColsTree; ++b) v[b] = {b < RB ? __ldcg(partials + b * N + j) : 0.f, 0.f};
 #pragma unroll
   for (int o = kColsTree / 2; o > 0; o >>= 1)
 #pragma unroll
-    for (int b = 0; b < o; ++b) v[b] = __fadd_rn(v[b], v[b + o]);
-  const float z = __fmul_rn(alpha, v[0]);
+    for (int b = 0; b < o; ++b) v[b] = comp_merge(v[b], v[b + o]);
+  const float z = __fmul_rn(alpha, comp_value32(v[0]));
   y[j] = beta == 0.f ? z : __fadd_rn(z, __fmul_rn(beta, y[j]));
 }
 

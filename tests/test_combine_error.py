@@ -1,0 +1,54 @@
+"""The combines of partial sums in the kernel expressions carry their rounding
+errors: adding fp32 partials costs one rounding of the result, however many
+partials there are and in whichever order a kernel adds them.
+
+With one row per block and x = 1 the partials are the matrix's own entries,
+so the exact sum is known.  A pair (sum, compensation) that goes through every add leaves the
+final rounding, u |S|, and second-order terms: at most m adds, each of whose
+errors is added to the compensation with one rounding, (m u)^2 sum|t|
+doubled as for a compensated sum."""
+import math
+
+import numpy as np
+import pytest
+
+from oracle import blas
+from oracle import lowlevel as ll
+from oracle.patterns import TreeComp, evaluate
+
+U = blas.U_FP32
+
+
+def columns(m, n, seed):
+    """m x n values of mixed sign and magnitude, exactly fp32."""
+    rng = np.random.default_rng(seed)
+    return (rng.standard_normal((m, n)) * 2.0 ** rng.integers(-3, 4, (m, n))).astype(np.float32)
+
+
+def sums(A, axis):
+    return np.array([math.fsum(v) for v in np.moveaxis(A.astype(np.float64), axis, -1)])
+
+
+@pytest.mark.parametrize("passes,cluster", [(1, 1), (2, 1)])
+@pytest.mark.parametrize("RB", [2, 31, 32, 33, 94, 512])
+def test_gemv_t_block_combine(RB, passes, cluster):
+    A = columns(RB, 200, RB)
+    z = evaluate(ll.gemv_t_z_variant(RB, 200, 1.0, 1, RB, passes, cluster), A, mode="f32",
+                 env={"x": np.ones(RB, np.float32)})
+    exact = sums(A, 0)
+    tol = U * np.abs(exact) + 2 * (RB * U) ** 2 * np.abs(A.astype(np.float64)).sum(0)
+    assert np.all(np.abs(z.astype(np.float64) - exact) <= tol)
+
+
+def test_tree_comp_values():
+    # 1 and 63 terms of 2^-24, one per lane: a plain fp32 tree loses terms
+    x = np.full((64, 1), 2.0 ** -24, np.float32)
+    x[0] = 1.0
+    assert evaluate(TreeComp(), x, mode="f32")[0] == np.float32(1 + 63 * 2.0 ** -24)
+    i = np.arange(64 * 5).reshape(64, 5)
+    assert evaluate(TreeComp(), i, mode="int")[0] == i.sum()
+    for v in (np.inf, -np.inf, np.nan):              # non-finite sums stay what they are
+        x[40] = v
+        assert np.array_equal(evaluate(TreeComp(), x, mode="f32"), [v], equal_nan=True)
+    x[41] = np.inf                                   # NaN + Inf
+    assert np.isnan(evaluate(TreeComp(), x, mode="f32")[0])
