@@ -216,20 +216,25 @@ def reduce_variant(op: str, n: int, tile: int, vw: int, threads: int, grid: int,
 GEMV_GROUP = 8   # vectors a gemv lane folds plainly before a compensated add
 
 
-def grouped_dot(vw: int, J: int, group: int = GEMV_GROUP):
-    """[J] zipped vectors of one lane -> [1]: groups of ``group``
+def group_values(vw: int, J: int, group: int = GEMV_GROUP):
+    """[J] zipped vectors of one lane -> [groups]: groups of ``group``
     consecutive vectors (the last padded with zeros), each folded from zero
-    over the vw lanes with its lanes then added in order, and the group
-    values added with the compensated reduce-seq (the partial reduction of
-    Fig. 3d applied to the lane's reduce-seq, its outer level
-    compensated)."""
+    over the vw lanes with its lanes then added in order."""
     f = fold(add, mult)
     fr = Vect(vw, f) if vw > 1 else f
     value = ReduceSeq(fr, 0)
     if vw > 1:
         value = C(ReduceSeq(add, 0), AsScalar(), ReduceSeq(fr, 0))
     Jp = max(group, math.ceil(J / group) * group)
-    return C(ReduceSeqComp(add), Join(), Map(value), Split(group), PadTo(Jp))
+    return C(Join(), Map(value), Split(group), PadTo(Jp))
+
+
+def grouped_dot(vw: int, J: int, group: int = GEMV_GROUP):
+    """[J] zipped vectors of one lane -> [1]: its group values (see
+    ``group_values``) added with the compensated reduce-seq (the partial
+    reduction of Fig. 3d applied to the lane's reduce-seq, its outer level
+    compensated)."""
+    return C(ReduceSeqComp(add), group_values(vw, J, group))
 
 
 def partials_combine(P: int):
@@ -265,15 +270,15 @@ def gemv_z_variant(M: int, N: int, alpha, vw: int, lanes: int = WARP,
 def gemv_split_z_variant(M: int, N: int, alpha, vw: int, threads: int, L: int, S: int):
     """z of the split-row gemv: each row zipped with x, padded to S*L and
     split into S segments of L elements; a CTA of ``threads`` folds a
-    segment (thread t takes vectors t, t+threads, ... in order and folds
-    them with ``grouped_dot``, then ``block_tree``); the S segment partials
-    of the row go through
+    segment (thread t takes vectors t, t+threads, ... in order, adds their
+    ``group_values`` compensated, and the threads' pairs go through the CTA's
+    trees: tree-comp); the S segment partials of the row go through
     ``partials_combine`` and the result is multiplied by alpha -- the
     partial-reduction rule of Fig. 3 applied to each row's reduce."""
     chunk = threads * vw
     assert L % chunk == 0 and S * L >= N
     J = L // chunk
-    segment = C(block_tree(threads), Join(), MapLocal(grouped_dot(vw, J)),
+    segment = C(TreeComp(), MapLocal(group_values(vw, J)),
                 Split(J), ReorderStride(s=threads), AsVector(vw) if vw > 1 else Id())
     row = C(Join(), MapWorkgroup(partials_combine(S)), Split(S), Join(), MapWorkgroup(segment),
             Split(L), PadTo(S * L), ZipWith("x"))

@@ -46,6 +46,50 @@ __device__ __forceinline__ Comp warp_comp(Comp v) {
   return v;
 }
 
+// The same for R rows at once (R a power of two): at each of the first
+// log2(R) levels a lane gives half of its rows to its partner and keeps the
+// other half, so R rows take R - 1 merges and the rest of one tree instead of
+// R trees.  Merges commute, so the bits are warp_comp's.  Row r's value ends
+// in lane r * (32 / R).
+template <int R>
+__device__ __forceinline__ Comp warp_comp_rows(Comp (&v)[R]) {
+  const int lane = threadIdx.x & (kWarp - 1);
+#pragma unroll
+  for (int n = R / 2, o = kWarp / 2; n > 0; n /= 2, o /= 2) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int k = 0; k < n; ++k) {
+      const Comp keep = up ? v[k + n] : v[k], give = up ? v[k] : v[k + n];
+      Comp w;
+      w.s = __shfl_xor_sync(0xffffffffu, give.s, o);
+      w.c = __shfl_xor_sync(0xffffffffu, give.c, o);
+      v[k] = comp_merge(keep, w);
+    }
+  }
+#pragma unroll
+  for (int o = kWarp / 2 / R; o > 0; o >>= 1) {
+    Comp w;
+    w.s = __shfl_down_sync(0xffffffffu, v[0].s, o);
+    w.c = __shfl_down_sync(0xffffffffu, v[0].c, o);
+    v[0] = comp_merge(v[0], w);
+  }
+  return v[0];
+}
+
+// The last levels of the tree, over lanes 0 .. N-1 (zeros above them would
+// change nothing).  Valid in lane 0.
+template <int N>
+__device__ __forceinline__ Comp warp_comp_first(Comp v) {
+#pragma unroll
+  for (int o = N / 2; o > 0; o >>= 1) {
+    Comp w;
+    w.s = __shfl_down_sync(0xffffffffu, v.s, o);
+    w.c = __shfl_down_sync(0xffffffffu, v.c, o);
+    v = comp_merge(v, w);
+  }
+  return v;
+}
+
 template <int THREADS>
 __device__ __forceinline__ Comp block_comp(Comp v) {
   __shared__ float rs[kWarp], rc[kWarp];

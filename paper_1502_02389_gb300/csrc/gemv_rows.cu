@@ -2,6 +2,10 @@
 // the same per-row expressions as the warp-per-row kernel of scal_gemv.cu
 // and the split-row kernel of gemv_split.cu).
 //
+// A row's sum is spread over more threads than the 32 lanes of a warp, so the
+// trees over them keep the compensations: the error of a row is no larger
+// than the warp-per-row kernel's.
+//
 // Both older forms load one vector of x for every vector of A, and give a
 // row to one warp or CTA at a time.  Here a warp (WARPS form) or a CTA
 // (split form) folds R consecutive rows together: a vector of x is loaded
@@ -23,7 +27,7 @@
 // The last, partial step of a row is read with guarded loads of all U
 // vectors at once (zeros past the end, which change nothing), so a ragged
 // row costs one more step instead of up to U dependent ones.
-#include "lift_internal.cuh"
+#include "comp_sum.cuh"
 
 namespace lift {
 
@@ -114,7 +118,7 @@ __global__ void __launch_bounds__(THREADS)
                     int64_t S, float* __restrict__ partials) {
   constexpr int W = THREADS / kWarp;
   static_assert(R <= W, "one warp per row in the last stage of the tree");
-  __shared__ float red[R][kWarp];
+  __shared__ Comp red[R][kWarp];
   const int lane = threadIdx.x & (kWarp - 1), warp = threadIdx.x / kWarp;
   const int64_t r0 = blockIdx.x / S * R, seg = blockIdx.x % S;
   const int64_t c_end = (seg + 1) * L < N ? (seg + 1) * L : N;
@@ -130,14 +134,17 @@ __global__ void __launch_bounds__(THREADS)
   for (int r = 0; r < R; ++r) acc[r].init();
   fold_r_rows<VW, R, U, THREADS * VW>(a, x, seg * L + (int64_t)threadIdx.x * VW, c_end, acc);
   pdl_trigger();   // streaming done: the combine kernel (or the next call's) may be scheduled
+  Comp v[R];
 #pragma unroll
   for (int r = 0; r < R; ++r) {
-    const float v = warp_tree(acc[r].value());
-    if (lane == 0) red[r][warp] = v;
+    acc[r].close();
+    v[r] = {acc[r].s, acc[r].c};
   }
+  const Comp mine = warp_comp_rows<R>(v);
+  if (lane % (kWarp / R) == 0) red[lane / (kWarp / R)][warp] = mine;
   __syncthreads();
   if (warp >= R || r0 + warp >= M) return;
-  const float d = warp_tree(lane < W ? red[warp][lane] : 0.0f);
+  const float d = comp_value32(warp_comp_first<W>(red[warp][lane % W]));
   if (lane != 0) return;
   if (S > 1) {
     partials[(r0 + warp) * S + seg] = d;

@@ -16,10 +16,12 @@
 // its VW lanes, and the CTA's halving tree (warp trees, then one warp over the
 // warp results) gives the segment partial.  COMBINE is the warp-per-row fold
 // of the S partials (lane l adds partials l, l+32, ..., then a halving tree
-// over the lanes), run by the programmatically dependent second kernel that
+// over the lanes).  Both trees add (sum, compensation) pairs, so that a row
+// spread over 128 or 256 threads and S CTAs is no less accurate than one
+// folded by the 32 lanes of a warp.  COMBINE is run by the programmatically dependent second kernel that
 // gemv-T uses; with S == 1 the CTA applies the epilogue itself.  The
 // epilogue is fl(fl(alpha * d) + fl(beta * y_r)) (y not read when beta == 0).
-#include "lift_internal.cuh"
+#include "comp_sum.cuh"
 
 namespace lift {
 
@@ -53,7 +55,6 @@ __global__ void __launch_bounds__(THREADS)
                const float* __restrict__ x, float beta, float* __restrict__ y, int64_t L,
                int64_t S, float* __restrict__ partials) {
   constexpr int64_t kStep = (int64_t)THREADS * VW;
-  __shared__ float red[kWarp];
   const int64_t r = blockIdx.x / S, seg = blockIdx.x % S;
   const int64_t c_end = (seg + 1) * L < N ? (seg + 1) * L : N;
   static_assert(kGemvGroup % U == 0, "an unrolled step stays inside one group");
@@ -86,7 +87,8 @@ __global__ void __launch_bounds__(THREADS)
     ld_guarded<VW>(x, c, c_end, b);
     acc.add(a, b);
   }
-  float d = block_tree<THREADS>(acc.value(), red);
+  acc.close();
+  const float d = comp_value32(block_comp<THREADS>({acc.s, acc.c}));
   if (S > 1) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (threadIdx.x != 0) return;
   if (S > 1) {

@@ -279,6 +279,11 @@ struct GroupedDot {
     flush();
     return neumaier_value(s, c);
   }
+  // the same, left as a sum and its compensation in s and c
+  __device__ __forceinline__ void close() {
+    if (!closed) s = lanes();
+    else flush();
+  }
 };
 
 // Halving tree over the 32 lanes of a warp: at offset o lane j adds lane

@@ -2,8 +2,9 @@
 errors: adding fp32 partials costs one rounding of the result, however many
 partials there are and in whichever order a kernel adds them.
 
-With one row per block and x = 1 the partials are the matrix's own entries,
-so the exact sum is known.  A pair (sum, compensation) that goes through every add leaves the
+With one row per block (gemv-T) or one element per thread (split-row gemv)
+and x = 1 the partials are the matrix's own entries, so the exact sum is
+known.  A pair (sum, compensation) that goes through every add leaves the
 final rounding, u |S|, and second-order terms: at most m adds, each of whose
 errors is added to the compensation with one rounding, (m u)^2 sum|t|
 doubled as for a compensated sum."""
@@ -37,6 +38,19 @@ def test_gemv_t_block_combine(RB, passes, cluster):
                  env={"x": np.ones(RB, np.float32)})
     exact = sums(A, 0)
     tol = U * np.abs(exact) + 2 * (RB * U) ** 2 * np.abs(A.astype(np.float64)).sum(0)
+    assert np.all(np.abs(z.astype(np.float64) - exact) <= tol)
+
+
+@pytest.mark.parametrize("threads,S", [(128, 1), (256, 1), (128, 2), (256, 40), (128, 94)])
+def test_gemv_split_row_combine(threads, S):
+    N = threads * S
+    A = columns(64, N, threads + S)
+    z = evaluate(ll.gemv_split_z_variant(64, N, 1.0, 1, threads, threads, S), A, mode="f32",
+                 env={"x": np.ones(N, np.float32)})
+    exact = sums(A, 1)
+    parts = np.abs(A.astype(np.float64).reshape(64, S, threads).sum(2)).sum(1) if S > 1 else 0.0
+    tol = U * (np.abs(exact) + 1.01 * parts) + \
+        2 * ((threads + S) * U) ** 2 * np.abs(A.astype(np.float64)).sum(1)
     assert np.all(np.abs(z.astype(np.float64) - exact) <= tol)
 
 
