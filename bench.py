@@ -706,7 +706,7 @@ def run_ours(args, rank, world, dist):
         vg = lift.lift_pick(op, M * N, M, N)
         pg = lift.lift_variant_describe(op, vg)
         if trans:
-            launches_per_step = pg["passes"]
+            launches_per_step = min(pg["passes"], 2)      # 3 and 4: two launches
         else:
             launches_per_step = 1 if lift.lift_gemv_segments(vg, M, N)[1] == 1 else 2
         bytes_step = 4 * M * N + 4 * nx + 8 * ny

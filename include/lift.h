@@ -328,7 +328,10 @@ lift_status lift_gemv_v(int variant, int64_t M, int64_t N, float alpha, const fl
  *           distribution (0 erfcf, 1 polynomial, 2 polynomial on
  *           approximate instructions)
  *  cluster  CTAs per cluster (1 = none)
- *  passes   1: last-CTA combine in the same launch; 2: second kernel
+ *  passes   1: last-CTA combine in the same launch; 2: second kernel;
+ *           3, 4 (gemv-T): second kernel, and the rows of a block folded
+ *           in shorter groups between compensated adds (16 instead of 32; 4:
+ *           pairs in blocks of 5 to 40 rows)
  *  stages   0: direct vector loads; k >= 2: k-deep TMA bulk-copy ring
  *  rows     gemv: rows per warp-group step; gemv-T, compensated, mixed
  *           precision, BlackScholes: loads (rows) in flight per work-item

@@ -286,18 +286,20 @@ def gemv_split_z_variant(M: int, N: int, alpha, vw: int, threads: int, L: int, S
 
 
 def gemv_t_z_variant(M: int, N: int, alpha, B: int, RB: int, passes: int = 1,
-                     cluster: int = 1, group: int = 32):
+                     cluster: int = 1):
     """z of the gemv-T kernel: every column of A (the rows of the
     reorder-stride view) zipped with x, padded to RB*B, folded in RB blocks
-    of B rows (fp32; a block's rows in groups of ``group``, each group
-    folded from zero, the group sums added with the compensated reduce-seq);
+    of B rows (fp32; a block's rows in groups of 32, each group folded from
+    zero, the group sums added with the compensated reduce-seq);
     the block partials are then combined in fp32 --
     one pass: added in block order with the compensated reduce-seq; one pass
     with clusters of ``cluster`` blocks: each cluster's consecutive block
     partials added in order, then the cluster sums added in order with the
     compensated reduce-seq (the partial reduction of Fig. 3d applied to the
     block partials); two pass: ``partials_combine``, one warp per column --
-    and multiplied by alpha."""
+    and multiplied by alpha.  passes = 3 and 4 are the two-pass form with
+    shorter groups: of 16 rows, with 4 of 2 rows in blocks of 5 to 40."""
+    group = 32 if passes < 3 else 2 if passes == 4 and 4 < B <= 40 else 16
     if passes == 1 and cluster > 1:
         assert RB % cluster == 0
         combine = C(ReduceSeqComp(add), Join(), Map(ReduceSeq(add, 0)), Split(cluster))

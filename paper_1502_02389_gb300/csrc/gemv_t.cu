@@ -176,34 +176,50 @@ __global__ void __launch_bounds__(THREADS)
 }
 
 // Second pass: column j's RB partials P[j][0..RB) -> y_j.  Warp w of the
-// grid takes columns w, w + W, ...; lane l folds partials l, l+32, ...
-// (eight loads in flight, added in order with Neumaier's compensated step),
-// then a halving tree over the lanes (shuffle-down 16, 8, 4, 2, 1) that keeps
-// the compensations: with lane values rounded before a plain tree, a column
-// of 94 block partials had 12 % more error than with the one-pass forms.
+// grid takes columns C*w .. C*w+C-1, and so on; lane l folds a column's
+// partials l, l+32, ... (added in order with Neumaier's compensated step),
+// then a halving tree over the lanes (shuffle 16, 8, 4, 2, 1) that keeps the
+// compensations: with lane values rounded before a plain tree, a column of
+// 94 block partials had 12 % more error than with the one-pass forms.  C
+// columns share one tree where a lane has few partials of each: C = 4 up to
+// kShareBlocks blocks (gemv-T of 500 x 6000: 6.8 us, 7.8 with a tree per
+// column; 2400 x 16384: 27.6, 29.5).  With more blocks the warps are too few
+// for the loads (65536 x 1024: 42.2 us, 42.6 with C = 4 up to 128 blocks).
+template <int C>
 __global__ void __launch_bounds__(256)
     gemv_t_combine(int64_t N, int64_t RB, float alpha, float beta,
                    const float* __restrict__ partials, float* __restrict__ y) {
   pdl_trigger();   // the next call's first kernel may be scheduled (it waits for this one)
   pdl_wait();      // the first pass has finished
+  constexpr int U = 8 / C;
   const int lane = threadIdx.x & (kWarp - 1);
-  const int64_t W = (int64_t)gridDim.x * (blockDim.x / kWarp);
-  for (int64_t j = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / kWarp; j < N; j += W) {
-    const float* p = partials + j * RB;
-    float s = 0.f, c = 0.f;              // the lane's partials in order, compensated
-    int64_t q = lane;
-    for (; q + 7 * kWarp < RB; q += 8 * kWarp) {
-      float v[8];
+  const int64_t W = (int64_t)gridDim.x * (blockDim.x / kWarp) * C;
+  for (int64_t j = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / kWarp * C; j < N; j += W) {
+    Comp v[C];
+    const float* p[C];
 #pragma unroll
-      for (int k = 0; k < 8; ++k) v[k] = __ldcg(p + q + k * kWarp);
-#pragma unroll
-      for (int k = 0; k < 8; ++k) neumaier_add(s, c, v[k]);
+    for (int k = 0; k < C; ++k) {
+      v[k] = {0.f, 0.f};
+      p[k] = partials + (j + k < N ? j + k : N - 1) * RB;
     }
-    for (; q < RB; q += kWarp) neumaier_add(s, c, __ldcg(p + q));
-    s = comp_value32(warp_comp({s, c}));
-    if (lane == 0) {
+    // eight loads in flight, the lane's partials of a column in order
+    for (int64_t q = lane; q - lane < RB; q += kWarp * U) {
+      float t[C][U];
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int k = 0; k < C; ++k) t[k][u] = q + u * kWarp < RB ? __ldcg(p[k] + q + u * kWarp) : 0.f;
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (q - lane + u * kWarp < RB)
+#pragma unroll
+          for (int k = 0; k < C; ++k) neumaier_add(v[k].s, v[k].c, t[k][u]);
+    }
+    const float s = comp_value32(warp_comp_rows<C>(v));
+    const int64_t col = j + lane / (kWarp / C);
+    if (lane % (kWarp / C) == 0 && col < N) {
       const float z = __fmul_rn(alpha, s);
-      y[j] = beta == 0.f ? z : __fadd_rn(z, __fmul_rn(beta, y[j]));
+      y[col] = beta == 0.f ? z : __fadd_rn(z, __fmul_rn(beta, y[col]));
     }
   }
 }
@@ -443,6 +459,7 @@ __global__ void __launch_bounds__(THREADS + kWarp, 1)
 }
 
 constexpr int kCombineThreads = 256;
+constexpr int64_t kShareBlocks = 64;
 constexpr int64_t kMaxRowBlocks2 = 512;   // two pass: at most 16 partials per lane
 
 constexpr int kTicketBase = 64;    // gemv-T tickets follow the reductions' counters
@@ -655,9 +672,11 @@ Variant gemv_t_variant(const char* name) {
 // the kernel before it on the stream.
 lift_status launch_rows_combine(int64_t n, int64_t per, float alpha, float beta,
                                 const float* partials, float* y, cudaStream_t s) {
-  const void* k = reinterpret_cast<const void*>(&gemv_t_combine);
-  const int64_t warps = kCombineThreads / kWarp;
-  int64_t g = (n + warps - 1) / warps;
+  const bool shared = per <= kShareBlocks;
+  const void* k = shared ? reinterpret_cast<const void*>(&gemv_t_combine<4>)
+                         : reinterpret_cast<const void*>(&gemv_t_combine<1>);
+  const int64_t outs = kCombineThreads / kWarp * (shared ? 4 : 1);   // per CTA
+  int64_t g = (n + outs - 1) / outs;
   const int64_t gmax = persistent_grid(k, kCombineThreads, 0, 1);
   if (g > gmax) g = gmax;
   if (g < 1) g = 1;

@@ -66,3 +66,22 @@ def test_tree_comp_values():
         assert np.array_equal(evaluate(TreeComp(), x, mode="f32"), [v], equal_nan=True)
     x[41] = np.inf                                   # NaN + Inf
     assert np.isnan(evaluate(TreeComp(), x, mode="f32")[0])
+
+
+# Row blocks (rows each, how many) of the one-pass form that 4-byte rows took
+# and of the form that they take, on a device of 152 SMs
+@pytest.mark.parametrize("M,old,new", [(40, 4, 8), (576, 4, 4), (689, 8, 12), (3147, 4, 8),
+                                       (9534, 8, 20), (4097, 44, 48), (8191, 216, 252),
+                                       (20000, 52, 60), (52140, 44, 104)])
+def test_gemv_t_of_4_byte_rows_is_no_less_accurate(M, old, new):
+    n = max(64, min(4096, (1 << 22) // M))
+    rng = np.random.default_rng(M)
+    A = rng.uniform(-1, 1, (M, n)).astype(np.float32)
+    x = rng.uniform(-1, 1, M).astype(np.float32)
+    exact = A.T.astype(np.float64) @ x.astype(np.float64)      # error far below fp32's
+    err = []
+    for B, passes in ((old, 1), (new, 4)):
+        z = evaluate(ll.gemv_t_z_variant(M, n, 1.0, B, -(-M // B), passes), A, mode="f32", env={"x": x})
+        err.append(np.linalg.norm(z.astype(np.float64) - exact))
+    # 2 %: the roundings of the products are the same in both, those of the sums are not
+    assert err[1] <= 1.02 * err[0]
