@@ -183,8 +183,9 @@ __global__ void __launch_bounds__(THREADS)
 // 94 block partials had 12 % more error than with the one-pass forms.  C
 // columns share one tree where a lane has few partials of each: C = 4 up to
 // kShareBlocks blocks (gemv-T of 500 x 6000: 6.8 us, 7.8 with a tree per
-// column; 2400 x 16384: 27.6, 29.5).  With more blocks the warps are too few
-// for the loads (65536 x 1024: 42.2 us, 42.6 with C = 4 up to 128 blocks).
+// column; 2400 x 16384: 27.6, 29.5) and from kShareOuts columns on.  With more
+// blocks or fewer columns the warps are too few for the loads (65536 x 1024:
+// 42.2 us, 42.6 with C = 4 up to 128 blocks; gemv of 64 x 32768: 4.2, 4.4).
 template <int C>
 __global__ void __launch_bounds__(256)
     gemv_t_combine(int64_t N, int64_t RB, float alpha, float beta,
@@ -459,7 +460,7 @@ __global__ void __launch_bounds__(THREADS + kWarp, 1)
 }
 
 constexpr int kCombineThreads = 256;
-constexpr int64_t kShareBlocks = 64;
+constexpr int64_t kShareBlocks = 64, kShareOuts = 2048;
 constexpr int64_t kMaxRowBlocks2 = 512;   // two pass: at most 16 partials per lane
 
 constexpr int kTicketBase = 64;    // gemv-T tickets follow the reductions' counters
@@ -672,7 +673,7 @@ Variant gemv_t_variant(const char* name) {
 // the kernel before it on the stream.
 lift_status launch_rows_combine(int64_t n, int64_t per, float alpha, float beta,
                                 const float* partials, float* y, cudaStream_t s) {
-  const bool shared = per <= kShareBlocks;
+  const bool shared = per <= kShareBlocks && n >= kShareOuts;
   const void* k = shared ? reinterpret_cast<const void*>(&gemv_t_combine<4>)
                          : reinterpret_cast<const void*>(&gemv_t_combine<1>);
   const int64_t outs = kCombineThreads / kWarp * (shared ? 4 : 1);   // per CTA
