@@ -378,6 +378,13 @@ static bool eligible(int op, const Variant& v, const Args& a) {
 //  * N < 2048: a warp per row, as the ring's stages would be mostly empty
 //    (20000 x 1024: 16.1 against 17; 80000 x 64: 16.9 against 44);
 //    8-float loads from 256 columns on, where one row fills a warp's load.
+//    A row of fewer than 2048 columns that ends inside a granule (N = 91, lda =
+//    92) was folded in 4-byte vectors before these rules, which leaves it 1 to
+//    9 % less error than 16-byte ones below 256 columns and from 512 on: it
+//    keeps them where they are as fast (80000 x 67: 13.0 us, 17.1 in 16-byte
+//    vectors; 7484 x 775: 8.1, 9.4; 30000 x 1351: 28, 30) and is split, whose
+//    trees keep the compensations, with fewer than 4000 rows (2000 x 1023:
+//    3.6, warp per row 6.4; 500 x 1023: 3.6, 2.6).
 //  * rows in 4-byte granules (N, lda or a pointer off 16 bytes): the forms
 //    that fold several rows at a time.  From 1024 columns on a CTA per row
 //    group (8193 x 5000: 29 against 62 for a warp per row), R = 4 rows where
@@ -399,8 +406,10 @@ static int fixed_gemv(const Args& a) {
   auto ok = [&](int k) { return eligible(LIFT_OP_GEMV, L[id[k]], a); };
   const int64_t M = a.M, N = a.N;
   if (ok(kWarp4)) {                     // 16-byte granules
-    if (N < 256) return id[kWarp4];
-    if (N < 2048) return id[ok(kWarp8) ? kWarp8 : kWarp4];
+    const bool whole = N % 4 == 0;
+    if (N < 256) return id[whole ? kWarp4 : kWarp1];
+    if (N < 2048 && (whole || N < 512)) return id[ok(kWarp8) ? kWarp8 : kWarp4];
+    if (N < 2048) return id[M < 4000 ? kSplit4 : N < 1024 ? kWarp1 : kSplit1Short];
     const bool few = N < 4096 ? M >= 1000 && M < 2000 : N < 8192 ? M >= 500 && M < 2000 : M < 2000;
     if (few) return id[kSplit4];
     const int ring = N < 4096 && M >= 2000 ? kRing4 : kRing;
