@@ -213,28 +213,30 @@ def reduce_variant(op: str, n: int, tile: int, vw: int, threads: int, grid: int,
     return e, L
 
 
-GEMV_GROUP = 8   # vectors a gemv lane folds plainly before a compensated add
-
-
-def group_values(vw: int, J: int, group: int = GEMV_GROUP):
-    """[J] zipped vectors of one lane -> [groups]: groups of ``group``
-    consecutive vectors (the last padded with zeros), each folded from zero
-    over the vw lanes with its lanes then added in order."""
+def group_values(vw: int, J: int):
+    """[J] zipped vectors of one lane -> [groups]: groups of 8 consecutive
+    vectors (4 of width 8; the last padded with zeros), each folded from zero
+    over the vw lanes with its lanes then added in order (8 lanes: in a
+    halving tree)."""
+    group = 4 if vw == 8 else 8
     f = fold(add, mult)
     fr = Vect(vw, f) if vw > 1 else f
     value = ReduceSeq(fr, 0)
     if vw > 1:
-        value = C(ReduceSeq(add, 0), AsScalar(), ReduceSeq(fr, 0))
+        lanes = ReduceSeq(add, 0)
+        if vw == 8:
+            lanes = Iterate(3, C(Join(), Map(lanes), Split(2), ReorderStride(n=2)))
+        value = C(lanes, AsScalar(), ReduceSeq(fr, 0))
     Jp = max(group, math.ceil(J / group) * group)
     return C(Join(), Map(value), Split(group), PadTo(Jp))
 
 
-def grouped_dot(vw: int, J: int, group: int = GEMV_GROUP):
+def grouped_dot(vw: int, J: int):
     """[J] zipped vectors of one lane -> [1]: its group values (see
     ``group_values``) added with the compensated reduce-seq (the partial
     reduction of Fig. 3d applied to the lane's reduce-seq, its outer level
     compensated)."""
-    return C(ReduceSeqComp(add), group_values(vw, J, group))
+    return C(ReduceSeqComp(add), group_values(vw, J))
 
 
 def partials_combine(P: int):
