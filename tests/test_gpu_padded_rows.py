@@ -31,10 +31,7 @@ def test_gemv(M, N, granule):
     ref = blas.gemv(A.astype(np.float64), x.astype(np.float64), y.astype(np.float64), 1.25, 0.5)
     tol = blas.tolerance(N, 1.0) * blas.gemv_row_terms(A, x, y, 1.25, 0.5)
     assert np.all(np.abs(yd.cpu().numpy().astype(np.float64) - ref) <= tol)
-<<<<<<< Updated upstream
     if N < 256 or (M >= 4000 and 512 <= N < 1024):       # rows folded in 4-byte vectors: variant 0's bits
         y0 = dev(y)
         L.lift_gemv_v(0, M, N, 1.25, Ad, lda, xd, 0.5, y0)
         assert torch.equal(yd, y0)
-=======
->>>>>>> Stashed changes
