@@ -45,6 +45,11 @@
  *    before another thread's call on that stream submits any).
  *    Calls on more than 8 streams at once share slots and can race (and
  *    after 4096 distinct stream handles the assignment starts afresh).
+ *    Beside the slot each of the first 256 streams of a device has scratch
+ *    of its own, which the fp32 asum, dot, nrm2 and sum and the gemv of few
+ *    rows use, so these do not race however many streams there are; on later
+ *    streams gemv runs forms that keep no scratch.  gemv-T, slices, and the
+ *    compensated and mixed-precision reductions use the slot.
  *  - Most kernels are launched as programmatic dependents of the kernel
  *    before them on the stream: their CTAs may be scheduled while that
  *    kernel still runs, but each waits for it to complete (and for its
@@ -111,8 +116,10 @@ typedef enum {
  * on it: 8 slots of partials and tickets (about 17 MiB each), one per
  * stream that launches work on the device (a stream takes the next slot on
  * its first call; beyond 8 streams slots are shared in turn), so calls on
- * up to 8 streams may run at the same time.  A CUDA graph keeps the slot of
- * the stream it was captured on.  Must be called (once per device) before
+ * up to 8 streams may run at the same time.  A CUDA graph keeps the slot and
+ * the scratch of the stream it was captured on, also those of its gemv calls:
+ * replays of graphs captured on one stream must not overlap on others.
+ * Must be called (once per device) before
  * any other call on that device, outside CUDA graph capture.  Calling it
  * again is a no-op; calls from several threads at once set the device up
  * once.

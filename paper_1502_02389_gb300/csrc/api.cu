@@ -62,11 +62,15 @@ DeviceState* current_state() {
 
 static Workspace& slot(DeviceState* st, int i) { return i == 0 ? st->ws : st->more[i - 1]; }
 
-// stream -> workspace slot, per device; a new stream takes the next slot
-static std::map<std::pair<DeviceState*, cudaStream_t>, int> g_slot_of;
+// stream -> workspace slot and scratch of its own, per device; a new stream
+// takes the next slot
+struct StreamScratch {
+  int slot, own;
+};
+static std::map<std::pair<DeviceState*, cudaStream_t>, StreamScratch> g_slot_of;
 static std::map<DeviceState*, int> g_next_slot;
 
-Workspace* stream_workspace(DeviceState* st, cudaStream_t stream) {
+Workspace* stream_workspace(DeviceState* st, cudaStream_t stream, int* own) {
   std::lock_guard<std::mutex> lk(g_mu);
   auto key = std::make_pair(st, stream);
   auto it = g_slot_of.find(key);
@@ -75,10 +79,13 @@ Workspace* stream_workspace(DeviceState* st, cudaStream_t stream) {
     // assignments once there are many (slots are then dealt afresh)
     if (g_slot_of.size() >= 4096) g_slot_of.clear();
     int& nx = g_next_slot[st];
-    it = g_slot_of.emplace(key, nx).first;
+    // (the per-thread default stream is one handle for many streams)
+    const bool one = stream != cudaStreamPerThread && st->owned < kOwnStreams;
+    it = g_slot_of.emplace(key, StreamScratch{nx, one ? st->owned++ : -1}).first;
     nx = (nx + 1) % kWsSlots;
   }
-  return &slot(st, it->second);
+  if (own) *own = it->second.own;
+  return &slot(st, it->second.slot);
 }
 
 static void free_slots(DeviceState* st) {
@@ -89,6 +96,8 @@ static void free_slots(DeviceState* st) {
     cudaFree(w.tickets);
     w = Workspace();
   }
+  cudaFree(st->own);
+  cudaFree(st->own_tickets);
 }
 
 // Serialises whole initialisations, so two threads that call lift_init for
@@ -128,6 +137,11 @@ static lift_status init_device(int device) {
     w.capacity = kPartialCapacity;
     w.capacity64 = kPartial64Capacity;
   }
+  const size_t own_tickets = kOwnStreams * kOwnTicketStride * sizeof(unsigned);
+  if (rc == LIFT_OK)
+    rc = cuda_check(cudaMalloc(&st->own, kOwnStreams * kOwnFloats * sizeof(float)), "workspace");
+  if (rc == LIFT_OK) rc = cuda_check(cudaMalloc(&st->own_tickets, own_tickets), "workspace");
+  if (rc == LIFT_OK) rc = cuda_check(cudaMemset(st->own_tickets, 0, own_tickets), "memset");
   if (rc == LIFT_OK) rc = cuda_check(cudaDeviceSynchronize(), "init sync");
   if (rc != LIFT_OK) {
     free_slots(st);
@@ -405,19 +419,26 @@ static int fixed_gemv(const Args& a) {
   const auto& L = registry(LIFT_OP_GEMV);
   auto ok = [&](int k) { return eligible(LIFT_OP_GEMV, L[id[k]], a); };
   const int64_t M = a.M, N = a.N;
+  // a stream that would share its scratch with another: a split row (more than
+  // one CTA of `rows` rows each) only where the forms before it had one
+  auto split = [&](int k, int rows, int otherwise) {
+    const bool alone = !a.must_share || L[id[k]].grid(L[id[k]], a) <= (M + rows - 1) / rows;
+    return id[alone ? k : otherwise];
+  };
   if (ok(kWarp4)) {                     // 16-byte granules
     const bool whole = N % 4 == 0;
     if (N < 256) return id[whole ? kWarp4 : kWarp1];
     if (N < 2048 && (whole || N < 512)) return id[ok(kWarp8) ? kWarp8 : kWarp4];
-    if (N < 2048) return id[M < 4000 ? kSplit4 : N < 1024 ? kWarp1 : kSplit1Short];
+    if (N < 2048 && M < 4000) return split(kSplit4, 2, kWarp1);
+    if (N < 2048) return N < 1024 ? id[kWarp1] : split(kSplit1Short, 4, kWarp1);
     const bool few = N < 4096 ? M >= 1000 && M < 2000 : N < 8192 ? M >= 500 && M < 2000 : M < 2000;
-    if (few) return id[kSplit4];
     const int ring = N < 4096 && M >= 2000 ? kRing4 : kRing;
-    return id[ok(ring) ? ring : kSplit4];
+    if (few || !ok(ring)) return split(kSplit4, 2, ok(ring) ? ring : kWarp1);
+    return id[ring];
   }
   if (N < 1024) return id[kWarp1];
-  if (N >= 65536) return id[kSplit1R4];
-  return id[N < 4096 && M >= 4000 ? kSplit1Short : kSplit1R2];
+  if (N >= 65536) return split(kSplit1R4, 4, kWarp1);
+  return N < 4096 && M >= 4000 ? split(kSplit1Short, 4, kWarp1) : split(kSplit1R2, 2, kWarp1);
 }
 
 // gemv-T, the same way (us):
@@ -493,7 +514,8 @@ constexpr int64_t kOneLaunchMax = 1 << 20;
 
 // call: the pick is for a call on stream s (lift_pick asks without one)
 static int fixed_pick(int op, const Args& a, cudaStream_t s = nullptr, bool call = false) {
-  if (call && a.n <= kOneLaunchMax && one_launch(op) >= 0 && !capturing(s)) return one_launch(op);
+  if (call && a.n <= kOneLaunchMax && one_launch(op) >= 0 && !a.must_share && !capturing(s))
+    return one_launch(op);
   if (op == LIFT_OP_GEMV) return fixed_gemv(a);
   if (op == LIFT_OP_GEMV_T) return fixed_gemv_t(a);
   return fixed_default(op);
@@ -849,7 +871,13 @@ static lift_status run(int op, int variant, const Args& a0, void* stream) {
   if (!st) return set_error(LIFT_ERR_NOT_INITIALIZED, "lift_init was not called for this device");
   const cudaStream_t s = static_cast<cudaStream_t>(stream);
   Args a = a0;
-  a.ws = stream_workspace(st, s);
+  int own = -1;
+  a.ws = stream_workspace(st, s, &own);
+  a.must_share = own < 0;
+  if (own >= 0) {
+    a.own = st->own + own * kOwnFloats;
+    a.own_ticket = st->own_tickets + own * kOwnTicketStride;
+  }
   // A call of two launches leaves partials in the slot between them, and a
   // timing of candidates uses the slot on a stream of its own: another host
   // thread's call on this stream comes before or after all of it.
@@ -991,6 +1019,8 @@ int lift_read_status(int clear) {
     bool ok = cudaDeviceSynchronize() == cudaSuccess;
     for (int i = 0; i < kWsSlots && ok; ++i)
       ok = cudaMemset(slot(st, i).tickets, 0, kTicketSlots * sizeof(unsigned)) == cudaSuccess;
+    ok = ok && cudaMemset(st->own_tickets, 0, kOwnStreams * kOwnTicketStride * sizeof(unsigned)) ==
+                   cudaSuccess;
     ok = ok && cudaMemset(st->ws.status, 0, sizeof(int)) == cudaSuccess &&
          cudaDeviceSynchronize() == cudaSuccess;
     if (!ok) return LIFT_ERR_CUDA;

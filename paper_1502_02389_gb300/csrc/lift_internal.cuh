@@ -37,6 +37,13 @@ struct Workspace {
 // running at the same time on different streams do not share partials or
 // tickets.
 constexpr int kWsSlots = 8;
+// Small scratch of a stream's own beside its slot, for the first kOwnStreams
+// streams of a device: the partials of an fp32 reduction or of a gemv with
+// split rows, one per row and CTA at most (5472 on 152 SMs), and a ticket.  A
+// default gemv keeps no scratch that another stream writes, however many
+// streams there are.
+constexpr int kOwnStreams = 256;
+constexpr int64_t kOwnFloats = 8192, kOwnTicketStride = 32;
 
 struct DeviceState {
   int device = -1;
@@ -44,11 +51,15 @@ struct DeviceState {
   Workspace ws;                    // slot 0 (also the capacities and the status word)
   Workspace more[kWsSlots - 1];    // slots 1 ..
   std::mutex slot_mu[kWsSlots];    // the slots' mutexes
+  float* own = nullptr;            // kOwnStreams * kOwnFloats
+  unsigned* own_tickets = nullptr; // kOwnStreams * kOwnTicketStride, 0 between calls
+  int owned = 0;                   // streams that have scratch of their own
 };
 
 DeviceState* current_state();  // state of the current device, or nullptr
-// The workspace slot of `stream` on the current device (assigned on first use).
-Workspace* stream_workspace(DeviceState* st, cudaStream_t stream);
+// The workspace slot of `stream` on the current device (assigned on first use),
+// and the index of its own scratch, -1 without.
+Workspace* stream_workspace(DeviceState* st, cudaStream_t stream, int* own = nullptr);
 void noalloc_forget();          // drop lift_asum_noalloc's cached per-device addresses
 
 lift_status set_error(lift_status s, const std::string& msg);
@@ -70,6 +81,9 @@ struct Args {
   float* result = nullptr;         // reduction result
   double* result64 = nullptr;
   Workspace* ws = nullptr;         // the calling stream's workspace slot (set by the entry point)
+  float* own = nullptr;            // its own scratch, or nullptr (the same)
+  unsigned* own_ticket = nullptr;
+  bool must_share = false;         // a call on a stream without scratch of its own
   int64_t n = 0, M = 0, N = 0, lda = 0;
   float alpha = 0.f, beta = 0.f;
 };
@@ -85,6 +99,11 @@ struct Variant {
   int align_bytes;       // pointer alignment the vector/TMA form needs
   int fallback;          // id (same op) of the guarded scalar form, or -1
 };
+
+// Where a call leaves `count` fp32 partials between its launches.
+inline float* partials_for(const Args& a, int64_t count) {
+  return a.own && count <= kOwnFloats ? a.own : a.ws->partials;
+}
 
 std::vector<Variant>& registry(int op);
 int batch_pick(int op, int64_t n, int64_t M, int64_t N);   // the pick of a batched op
