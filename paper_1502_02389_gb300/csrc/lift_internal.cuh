@@ -170,16 +170,20 @@ struct Vec {
 };
 
 // Streaming loads: read-only path, no L1 allocation, 256-byte L2 prefetch.
+// volatile, as pdl_wait is: an asm that is neither volatile nor a memory
+// operation may be moved across the wait, and a kernel launched early would
+// read what the kernel before it has yet to write.  (No kernel's registers
+// changed with it.)
 __device__ __forceinline__ void ld_stream(const float* p, Vec<1>& o) {
-  asm("ld.global.nc.L1::no_allocate.L2::256B.f32 %0, [%1];" : "=f"(o.v[0]) : "l"(p));
+  asm volatile("ld.global.nc.L1::no_allocate.L2::256B.f32 %0, [%1];" : "=f"(o.v[0]) : "l"(p));
 }
 __device__ __forceinline__ void ld_stream(const float* p, Vec<4>& o) {
-  asm("ld.global.nc.L1::no_allocate.L2::256B.v4.f32 {%0,%1,%2,%3}, [%4];"
+  asm volatile("ld.global.nc.L1::no_allocate.L2::256B.v4.f32 {%0,%1,%2,%3}, [%4];"
       : "=f"(o.v[0]), "=f"(o.v[1]), "=f"(o.v[2]), "=f"(o.v[3])
       : "l"(p));
 }
 __device__ __forceinline__ void ld_stream(const float* p, Vec<8>& o) {
-  asm("ld.global.nc.L1::no_allocate.L2::256B.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+  asm volatile("ld.global.nc.L1::no_allocate.L2::256B.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
       : "=f"(o.v[0]), "=f"(o.v[1]), "=f"(o.v[2]), "=f"(o.v[3]), "=f"(o.v[4]), "=f"(o.v[5]),
         "=f"(o.v[6]), "=f"(o.v[7])
       : "l"(p));

@@ -55,13 +55,13 @@ struct Raw {
 
 __device__ __forceinline__ void ld_words(const uint32_t* p, uint32_t* w, int count) {
   for (int i = 0; i < count; i += 8)
-    asm("ld.global.nc.L1::no_allocate.L2::256B.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+    asm volatile("ld.global.nc.L1::no_allocate.L2::256B.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
         : "=r"(w[i]), "=r"(w[i + 1]), "=r"(w[i + 2]), "=r"(w[i + 3]), "=r"(w[i + 4]),
           "=r"(w[i + 5]), "=r"(w[i + 6]), "=r"(w[i + 7])
         : "l"(p + i));
 }
 __device__ __forceinline__ void ld_words4(const uint32_t* p, uint32_t* w) {
-  asm("ld.global.nc.L1::no_allocate.L2::256B.v4.b32 {%0,%1,%2,%3}, [%4];"
+  asm volatile("ld.global.nc.L1::no_allocate.L2::256B.v4.b32 {%0,%1,%2,%3}, [%4];"
       : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3])
       : "l"(p));
 }
