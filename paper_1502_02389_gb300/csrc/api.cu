@@ -97,7 +97,6 @@ static void free_slots(DeviceState* st) {
     w = Workspace();
   }
   cudaFree(st->own);
-  cudaFree(st->own_tickets);
 }
 
 // Serialises whole initialisations, so two threads that call lift_init for
@@ -137,11 +136,9 @@ static lift_status init_device(int device) {
     w.capacity = kPartialCapacity;
     w.capacity64 = kPartial64Capacity;
   }
-  const size_t own_tickets = kOwnStreams * kOwnTicketStride * sizeof(unsigned);
-  if (rc == LIFT_OK)
-    rc = cuda_check(cudaMalloc(&st->own, kOwnStreams * kOwnFloats * sizeof(float)), "workspace");
-  if (rc == LIFT_OK) rc = cuda_check(cudaMalloc(&st->own_tickets, own_tickets), "workspace");
-  if (rc == LIFT_OK) rc = cuda_check(cudaMemset(st->own_tickets, 0, own_tickets), "memset");
+  const size_t own_bytes = kOwnStreams * kOwnWords * sizeof(float);
+  if (rc == LIFT_OK) rc = cuda_check(cudaMalloc(&st->own, own_bytes), "workspace");
+  if (rc == LIFT_OK) rc = cuda_check(cudaMemset(st->own, 0, own_bytes), "memset");
   if (rc == LIFT_OK) rc = cuda_check(cudaDeviceSynchronize(), "init sync");
   if (rc != LIFT_OK) {
     free_slots(st);
@@ -875,8 +872,8 @@ static lift_status run(int op, int variant, const Args& a0, void* stream) {
   a.ws = stream_workspace(st, s, &own);
   a.must_share = own < 0;
   if (own >= 0) {
-    a.own = st->own + own * kOwnFloats;
-    a.own_ticket = st->own_tickets + own * kOwnTicketStride;
+    a.own = st->own + own * kOwnWords;
+    a.own_ticket = reinterpret_cast<unsigned*>(a.own + kOwnFloats);
   }
   // A call of two launches leaves partials in the slot between them, and a
   // timing of candidates uses the slot on a stream of its own: another host
@@ -1019,8 +1016,7 @@ int lift_read_status(int clear) {
     bool ok = cudaDeviceSynchronize() == cudaSuccess;
     for (int i = 0; i < kWsSlots && ok; ++i)
       ok = cudaMemset(slot(st, i).tickets, 0, kTicketSlots * sizeof(unsigned)) == cudaSuccess;
-    ok = ok && cudaMemset(st->own_tickets, 0, kOwnStreams * kOwnTicketStride * sizeof(unsigned)) ==
-                   cudaSuccess;
+    ok = ok && cudaMemset(st->own, 0, kOwnStreams * kOwnWords * sizeof(float)) == cudaSuccess;
     ok = ok && cudaMemset(st->ws.status, 0, sizeof(int)) == cudaSuccess &&
          cudaDeviceSynchronize() == cudaSuccess;
     if (!ok) return LIFT_ERR_CUDA;
