@@ -215,10 +215,9 @@ def reduce_variant(op: str, n: int, tile: int, vw: int, threads: int, grid: int,
 
 def group_values(vw: int, J: int):
     """[J] zipped vectors of one lane -> [groups]: groups of 8 consecutive
-    vectors (4 of width 8; the last padded with zeros), each folded from zero
-    over the vw lanes with its lanes then added in order (8 lanes: in a
-    halving tree)."""
-    group = 4 if vw == 8 else 8
+    vectors (the last padded with zeros), each folded from zero over the vw
+    lanes with its lanes then added in order (8 lanes: in a halving tree)."""
+    group = 8
     f = fold(add, mult)
     fr = Vect(vw, f) if vw > 1 else f
     value = ReduceSeq(fr, 0)

@@ -388,7 +388,12 @@ static bool eligible(int op, const Variant& v, const Args& a) {
 //    the ring: no second pass (64 x 4096: 3.0 against 3.5).
 //  * N < 2048: a warp per row, as the ring's stages would be mostly empty
 //    (20000 x 1024: 16.1 against 17; 80000 x 64: 16.9 against 44);
-//    8-float loads from 256 columns on, where one row fills a warp's load.
+//    8-float loads from 256 columns on, where one row fills a warp's load, to
+//    1279: beyond, their lanes fold more products plainly than 4-float ones
+//    and they are slower (30000 x 1352: 29.2 in 4-float loads, 30.7; 30000 x
+//    2040: 38.7, 45.0; 65536 x 1024: 44.3, 41.5); with fewer than 4000 of
+//    these rows they are split (1500 x 1352: 3.7, warp per row 5.4; 500 x
+//    2040: 4.5, 5.2; 500 x 1536: 4.0, 2.5).
 //    A row of fewer than 2048 columns that ends inside a granule (N = 91, lda =
 //    92) was folded in 4-byte vectors before these rules, which leaves it 1 to
 //    9 % less error than 16-byte ones below 256 columns and from 512 on: it
@@ -425,8 +430,9 @@ static int fixed_gemv(const Args& a) {
   if (ok(kWarp4)) {                     // 16-byte granules
     const bool whole = N % 4 == 0;
     if (N < 256) return id[whole ? kWarp4 : kWarp1];
-    if (N < 2048 && (whole || N < 512)) return id[ok(kWarp8) ? kWarp8 : kWarp4];
-    if (N < 2048 && M < 4000) return split(kSplit4, 2, kWarp1);
+    if (N < 512 || (whole && N < 1280)) return id[ok(kWarp8) ? kWarp8 : kWarp4];
+    if (N < 2048 && M < 4000) return split(kSplit4, 2, whole ? kWarp4 : kWarp1);
+    if (N < 2048 && whole) return id[kWarp4];
     if (N < 2048) return N < 1024 ? id[kWarp1] : split(kSplit1Short, 4, kWarp1);
     const bool few = N < 4096 ? M >= 1000 && M < 2000 : N < 8192 ? M >= 500 && M < 2000 : M < 2000;
     const int ring = N < 4096 && M >= 2000 ? kRing4 : kRing;

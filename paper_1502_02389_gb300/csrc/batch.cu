@@ -219,7 +219,7 @@ __device__ __forceinline__ void ld_x(const float* p, Vec<VW>& o) {
 template <int VW, int R, int U>
 __device__ __forceinline__ void gemv_item(const OpDev& o, int64_t r0, int64_t r1) {
   constexpr int kStep = kWarp * VW, kPiece = 1 << 28;
-  static_assert(kGemvGroup<VW> % U == 0 && kPiece % (kGemvGroup<VW> * kStep) == 0, "whole groups");
+  static_assert(kGemvGroup % U == 0 && kPiece % (kGemvGroup * kStep) == 0, "whole groups");
   const int lane = threadIdx.x & (kWarp - 1);
   for (int64_t row = r0 + threadIdx.x / kWarp * R; row < r1; row += kThreads / kWarp * R) {
     const int have = r1 - row < R ? (int)(r1 - row) : R;
@@ -248,7 +248,7 @@ __device__ __forceinline__ void gemv_item(const OpDev& o, int64_t r0, int64_t r1
         for (int u = 0; u < U; ++u)
 #pragma unroll
           for (int r = 0; r < R; ++r) acc[r].add(va[r][u], vx[u]);
-        k = (k + U) & (kGemvGroup<VW> - 1);
+        k = (k + U) & (kGemvGroup - 1);
         if (k == 0) {
 #pragma unroll
           for (int r = 0; r < R; ++r) acc[r].flush();

@@ -60,7 +60,7 @@ __device__ __forceinline__ void ld_x_rows(const float* p, Vec<VW>& o) {
 template <int VW, int R, int U, int STEP>
 __device__ __forceinline__ void fold_r_rows(const float* const (&a)[R], const float* x, int64_t c,
                                             int64_t c_end, GroupedDot<VW> (&acc)[R]) {
-  static_assert(kGemvGroup<VW> % U == 0, "an unrolled step stays inside one group");
+  static_assert(kGemvGroup % U == 0, "an unrolled step stays inside one group");
   int k = 0;                           // vectors folded (mod the group)
   for (; c + (int64_t)(U - 1) * STEP + VW <= c_end; c += (int64_t)U * STEP) {
     Vec<VW> v[R][U], b[U];
@@ -74,7 +74,7 @@ __device__ __forceinline__ void fold_r_rows(const float* const (&a)[R], const fl
     for (int u = 0; u < U; ++u)
 #pragma unroll
       for (int r = 0; r < R; ++r) acc[r].add(v[r][u], b[u]);
-    k = (k + U) & (kGemvGroup<VW> - 1);
+    k = (k + U) & (kGemvGroup - 1);
     if (k == 0) {
 #pragma unroll
       for (int r = 0; r < R; ++r) acc[r].flush();

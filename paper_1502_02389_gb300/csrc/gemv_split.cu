@@ -57,7 +57,7 @@ __global__ void __launch_bounds__(THREADS)
   constexpr int64_t kStep = (int64_t)THREADS * VW;
   const int64_t r = blockIdx.x / S, seg = blockIdx.x % S;
   const int64_t c_end = (seg + 1) * L < N ? (seg + 1) * L : N;
-  static_assert(kGemvGroup<VW> % U == 0, "an unrolled step stays inside one group");
+  static_assert(kGemvGroup % U == 0, "an unrolled step stays inside one group");
   const float* row = A + r * lda;
   GroupedDot<VW> acc;
   acc.init();
@@ -72,14 +72,14 @@ __global__ void __launch_bounds__(THREADS)
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) acc.add(a[u], b[u]);
-    if (((k + U) & (kGemvGroup<VW> - 1)) == 0) acc.flush();
+    if (((k + U) & (kGemvGroup - 1)) == 0) acc.flush();
   }
   for (; c + VW <= c_end; c += kStep, ++k) {
     Vec<VW> a, b;
     ld_stream(row + c, a);
     ld_x_vec<VW>(x + c, b);
     acc.add(a, b);
-    if (((k + 1) & (kGemvGroup<VW> - 1)) == 0) acc.flush();
+    if (((k + 1) & (kGemvGroup - 1)) == 0) acc.flush();
   }
   if (c < c_end) {           // the ragged last vector of the row
     Vec<VW> a, b;

@@ -107,8 +107,8 @@ __global__ void __launch_bounds__((WARPS + 1) * kWarp, 1)
   }
 
   // consumer warps: warp w folds row (block start + w); lane l's vectors of
-  // a row are l, l+32, ... (J per chunk), grouped kGemvGroup<4> at a time
-  static_assert(J % kGemvGroup<4> == 0 || kGemvGroup<4> % J == 0, "groups align with chunks");
+  // a row are l, l+32, ... (J per chunk), grouped kGemvGroup at a time
+  static_assert(J % kGemvGroup == 0 || kGemvGroup % J == 0, "groups align with chunks");
   GroupedDot<4> acc;
   acc.init();
   for (int64_t k = 0; k < total; ++k) {
@@ -135,12 +135,12 @@ __global__ void __launch_bounds__((WARPS + 1) * kWarp, 1)
           v = a;
         }
         acc.add(a, v);
-        if constexpr (J % kGemvGroup<4> == 0) {
-          if (((j + 1) & (kGemvGroup<4> - 1)) == 0) acc.flush();
+        if constexpr (J % kGemvGroup == 0) {
+          if (((j + 1) & (kGemvGroup - 1)) == 0) acc.flush();
         }
       }
-      if constexpr (J % kGemvGroup<4> != 0) {   // a group spans several chunks
-        if ((ch + 1) % (kGemvGroup<4> / J) == 0) acc.flush();
+      if constexpr (J % kGemvGroup != 0) {   // a group spans several chunks
+        if ((ch + 1) % (kGemvGroup / J) == 0) acc.flush();
       }
     }
     __syncwarp();

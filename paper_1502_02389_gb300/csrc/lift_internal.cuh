@@ -262,12 +262,10 @@ __device__ __forceinline__ float neumaier_value(float s, float c) {
 // form groups gG .. gG+G-1; a group's products are folded from zero over
 // the VW lanes, the lanes added in order (8 lanes: in a halving tree), and the
 // group values added with neumaier_add, so a row's error does not grow with
-// its length.  A power of two (it masks counters).  8-float vectors: half as
-// many, so that a group has the products of one of 4-float vectors, which rows
-// of 256 to 2047 columns were folded in before (813 x 256: relative l2 error
-// 8.8e-8 with 4-float vectors, 9.1e-8 with 8 vectors and the lanes in order).
-template <int VW>
-constexpr int kGemvGroup = VW == 8 ? 4 : 8;
+// its length.  (Eight lanes in order gave 813 x 256 a relative l2 error of
+// 9.1e-8; in 4-float vectors, the form before, it has 8.8e-8.)
+constexpr int kGemvGroup = 8;   // a power of two
+static_assert((kGemvGroup & (kGemvGroup - 1)) == 0, "group masks need a power of two");
 
 template <int VW>
 struct GroupedDot {

@@ -340,7 +340,7 @@ __global__ void __launch_bounds__(WARPS * kWarp)
   const int64_t gw = (int64_t)blockIdx.x * WARPS + threadIdx.x / kWarp;
   const int64_t total = (int64_t)gridDim.x * WARPS;
   const int64_t chunks = N / kChunk;
-  static_assert(kGemvGroup<VW> % UNROLL == 0, "an unrolled step stays inside one group");
+  static_assert(kGemvGroup % UNROLL == 0, "an unrolled step stays inside one group");
   for (int64_t row = gw; row < M; row += total) {
     const float* a = A + row * lda;
     GroupedDot<VW> acc;
@@ -356,7 +356,7 @@ __global__ void __launch_bounds__(WARPS * kWarp)
       }
 #pragma unroll
       for (int u = 0; u < UNROLL; ++u) acc.add(va[u], vx[u]);
-      if (((c + UNROLL) & (kGemvGroup<VW> - 1)) == 0) acc.flush();
+      if (((c + UNROLL) & (kGemvGroup - 1)) == 0) acc.flush();
     }
     for (; c < chunks; ++c) {
       Vec<VW> va, vx;
@@ -364,7 +364,7 @@ __global__ void __launch_bounds__(WARPS * kWarp)
       ld_stream(a + e, va);
       ld_x<VW>(x + e, vx);
       acc.add(va, vx);
-      if (((c + 1) & (kGemvGroup<VW> - 1)) == 0) acc.flush();
+      if (((c + 1) & (kGemvGroup - 1)) == 0) acc.flush();
     }
     if (chunks * kChunk < N) {
       Vec<VW> va, vx;

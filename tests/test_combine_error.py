@@ -87,7 +87,7 @@ def test_gemv_t_of_4_byte_rows_is_no_less_accurate(M, old, new):
     assert err[1] <= 1.02 * err[0]
 
 
-@pytest.mark.parametrize("N", [256, 320, 512, 776, 1024, 1536, 2040])
+@pytest.mark.parametrize("N", [256, 320, 512, 776, 1024, 1272])
 def test_gemv_rows_of_8_float_vectors_are_no_less_accurate(N):
     # against the 4-float vectors that such rows were read in before; six
     # matrices, whose errors differ by 1 to 6 % and scatter by 1 % each
