@@ -36,8 +36,12 @@
  *  - A pointer that is not aligned for a variant's vector width or for
  *    TMA bulk copies (16 B) makes the library use the same variant family's
  *    guarded scalar-load form instead; it is not an error.  A vector op
- *    called without a variant id reads slices that start off a 16-byte
- *    boundary in 16-byte loads all the same.
+ *    called without a variant id whose pick needs an alignment that the
+ *    pointers lack (under the FIXED policy, every slice that starts off a
+ *    16-byte boundary; the learned policies pick a 4-byte variant for it)
+ *    reads it in 16-byte loads all the same.  A reduction's tiles are then
+ *    split from the boundary below the slice, so its bits depend on the
+ *    slice's offset from there (scal and axpy are elementwise).
  *  - The reductions use a per-device workspace allocated by lift_init
  *    (partials, ticket counters, a status word), one slot per stream for up
  *    to 8 streams of a device; calls on the same stream are ordered by it,

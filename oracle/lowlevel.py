@@ -213,6 +213,31 @@ def reduce_variant(op: str, n: int, tile: int, vw: int, threads: int, grid: int,
     return e, L
 
 
+UNALIGNED_TILE = 4096   # 256 threads x 4 vectors of 4
+
+
+def unaligned_reduce(op: str, n: int, m: int, grid: int, cast32: bool = True):
+    """Expression of a default reduction of a slice that starts m elements
+    past a 16-byte boundary, and the length of its input: m zeros, the n
+    elements, zeros.  The tiles are split from the boundary; in a tile each
+    warp takes 128 consecutive vectors, lane l vectors l, l+32, l+64, l+96 of
+    them; tiles, trees and combine as in ``reduce_variant``."""
+    T = max(1, math.ceil((n + m) / UNALIGNED_TILE))
+    K = math.ceil(T / grid)
+    f = FOLD[op]
+    tile_value = C(ReduceSeq(add, 0), AsScalar(), ReduceSeq(Vect(4, f), 0))
+    per_thread = C(ReduceSeqComp(add), Join(), Map(tile_value), Split(4))
+    order = C(_thread_order(256, K * 4, 4, False), Join(), Map(ReorderStride(s=WARP)), Split(4 * WARP))
+    cta = C(block_tree(256), Join(), MapLocal(per_thread), order, AsVector(4))
+    L = grid * K * UNALIGNED_TILE
+    e = C(final_combine(grid, 256, cast32, sqrt64 if op == "nrm2" else None),
+          Join(), MapWorkgroup(cta), Split(K * UNALIGNED_TILE), Join(),
+          ReorderStride(s=grid), Split(UNALIGNED_TILE), PadTo(L))
+    if op == "dot":
+        e = C(e, Zip())
+    return e, L
+
+
 def group_values(vw: int, J: int):
     """[J] zipped vectors of one lane -> [groups]: groups of 8 consecutive
     vectors (the last padded with zeros), each folded from zero over the vw
