@@ -159,6 +159,7 @@ __global__ void __launch_bounds__(kLossThreads)
 // ---------------------------------------------------------------------------
 constexpr int kH = 64;               // hidden units
 constexpr int kRows = 16;            // rows of the batch per CTA
+constexpr int kMaxShared = 227 * 1024;   // bytes a CTA may have: with it one CTA fits an SM
 constexpr int kPitch = 20;           // floats between columns of a [.][kRows] array in shared
                                      // memory: 16-byte rows, 4-way conflicts at most on writes
 
@@ -220,8 +221,10 @@ __device__ __forceinline__ void hidden_layer(int K, const float* in, const float
 // memory at once (85 KB for 265 outputs), W3 while the hidden layers run.
 // The last layer gives a thread one output column of all 16 rows: a weight
 // is read once and used 16 times against broadcast reads of the activations.
-// CW: columns of W3 staged at a time (all of them up to kFwdColumns).
-constexpr int kFwdColumns = 640;
+// CW: columns of W3 staged at a time (all of them up to kFwdColumns, what fits
+// the shared memory beside the other matrices).
+constexpr int kFwdColumns =
+    (kMaxShared / 4 - 2 * kH * kH - 2 * kH * kPitch) / kH / kWarp * kWarp;       // 736
 
 __global__ void __launch_bounds__(512)
     mlp_forward_fused(int B, int d, int V, int CW, const float* __restrict__ W1,
@@ -290,8 +293,14 @@ __global__ void __launch_bounds__(512)
 // per CTA.  W3 (in chunks of CW output columns) and W2 are staged in shared
 // memory with an odd pitch, so that 32 threads that walk 32 rows of W
 // together read 32 banks; the sum over a row's columns is split between four
-// quarters of the CTA.
+// quarters of the CTA.  A chunk is what fits the shared memory of an SM: a
+// batch of 2308 rows is 145 CTAs, one per SM whatever they hold, and its
+// copies are waited for once per chunk (both gradient launches, us: 2308 x 400
+// 30.0, in two chunks 37.1; 4096 x 512 57.8, 60.3; 3000 x 300, where two CTAs
+// of half a chunk would share an SM, 30.5, 29.7).
 constexpr int kActThreads = 512;
+constexpr int kBackColumns =
+    (kMaxShared / 4 - 6 * kH * kPitch - kH * (kH + 1) - kH) / (kPitch + kH) / kWarp * kWarp;   // 544
 
 // Thread (units j and j + 32, rows 4g .. 4g+3, a quarter of the columns): one
 // broadcast read of four rows serves two units.
@@ -392,7 +401,12 @@ __global__ void __launch_bounds__(kActThreads)
 // shares by thread (share, 8 consecutive i, c), and the shares added in order
 // through distributed shared memory.
 constexpr int kGradCtas = 8, kGradI = 8, kGradGroups = kH / kGradI, kGradShares = 4;
-constexpr int kGradThreads = kGradShares * kGradGroups * kWarp, kGradRows = 304;
+constexpr int kGradThreads = kGradShares * kGradGroups * kWarp;
+// rows of L and R that fit the shared memory of an SM beside the sums: 512
+// (4096 x 64: 27.7 us for both gradient launches, 28.5 in pieces of 304 rows)
+constexpr int kGradRowBytes = (kH + kWarp) * (int)sizeof(float);
+constexpr int kGradRows =
+    (kMaxShared - kGradShares * (kH + 1) * kWarp * (int)sizeof(float)) / kGradRowBytes / 16 * 16;
 
 struct GradJob {
   const float* L;      // rows x li
@@ -425,7 +439,7 @@ __global__ void __launch_bounds__(kGradThreads)
   pdl_trigger();   // the next launch may be scheduled (it waits for this one)
   pdl_wait();      // the launch before has finished
   if (li < kH)                                           // columns past L stay zero
-    for (int e = threadIdx.x; e < kGradRows * kH; e += kGradThreads)
+    for (int e = threadIdx.x; e < (b1 - b0 < kGradRows ? b1 - b0 : kGradRows) * kH; e += kGradThreads)
       if (e % kH >= li) ls[e] = 0.f;
   for (int r0 = b0; r0 < b1; r0 += kGradRows) {
     const int rows = b1 - r0 < kGradRows ? b1 - r0 : kGradRows;
@@ -576,7 +590,7 @@ lift_status forward_fused(int d, int V, const float* p, const Layout& L, const f
   threads = threads < 256 ? 256 : threads > 512 ? 512 : threads;
   const size_t smem = sizeof(float) * ((size_t)kH * CW + 2 * kH * kH + 2 * kH * kPitch);
   const lift_status rc = cuda_check(
-      cudaFuncSetAttribute(mlp_forward_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, 208 * 1024),
+      cudaFuncSetAttribute(mlp_forward_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxShared),
       "mlp_forward shared memory");
   if (rc != LIFT_OK) return rc;
   const float *W1 = p + L.W1, *b1 = p + L.b1, *W2 = p + L.W2, *b2 = p + L.b2, *W3 = p + L.W3,
@@ -589,13 +603,12 @@ lift_status forward_fused(int d, int V, const float* p, const Layout& L, const f
 lift_status backward_fused(int d, int V, const float* p, const Layout& L, const float* X, int B,
                            const float* H1, const float* H2, float* D0, float* D1, const float* dP,
                            float* grads, cudaStream_t s) {
-  constexpr int kChunk = 288;                        // output columns staged at a time, at most
-  const int chunks = (V + kChunk - 1) / kChunk, CW = (V + chunks - 1) / chunks;
+  const int chunks = (V + kBackColumns - 1) / kBackColumns, CW = (V + chunks - 1) / chunks;
   const size_t smem = sizeof(float) * ((size_t)CW * kPitch + 6 * kH * kPitch + kH * (kH + 1) +
                                        (size_t)kH * (CW | 1));
   lift_status rc = cuda_check(cudaFuncSetAttribute(mlp_back_rows,
                                                    cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   152 * 1024), "mlp_backward shared memory");
+                                                   kMaxShared), "mlp_backward shared memory");
   if (rc != LIFT_OK) return rc;
   const float *W2 = p + L.W2, *W3 = p + L.W3;
   void* rows_args[] = {&B, &V, const_cast<int*>(&CW), &W2, &W3, &H1, &H2, &dP, &D0, &D1};
@@ -607,7 +620,7 @@ lift_status backward_fused(int d, int V, const float* p, const Layout& L, const 
   GradJobs jobs = {{{H2, dP, grads + L.W3, grads + L.b3, kH, V, 0, hv},
                     {H1, D0, grads + L.W2, grads + L.b2, kH, kH, t3, hv},
                     {X, D1, grads + L.W1, grads + L.b1, d, kH, t3 + t64, xv}}};
-  constexpr int kGradSmem = kGradRows * (kH + kWarp) * (int)sizeof(float);
+  constexpr int kGradSmem = kGradRows * kGradRowBytes;
   rc = cuda_check(cudaFuncSetAttribute(mlp_weight_grads, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        kGradSmem), "mlp_backward shared memory");
   if (rc != LIFT_OK) return rc;
