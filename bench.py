@@ -423,7 +423,7 @@ def run_ours(args, rank, world, dist):
             calls.append((op, dt, dargs, v, lift.lift_variant_describe(op, v)["name"], nb))
         kernels = [["mixed:" + name, nb, [], []] for (_, _, _, _, name, nb) in calls]
         bytes_step = sum(c[5] for c in calls)
-        launches_per_step = 4
+        launches_per_step = 6          # the two sums add their partials in a second kernel
 
         def mixed_call(i):
             op, dt, da, v, name, nb = calls[i]
