@@ -57,8 +57,9 @@
  *  - Most kernels are launched as programmatic dependents of the kernel
  *    before them on the stream: their CTAs may be scheduled while that
  *    kernel still runs, but each waits for it to complete (and for its
- *    writes to be visible) before touching memory, so calls on one stream
- *    stay ordered exactly as stream order promises.
+ *    writes to be visible) before it reads or writes memory, so calls on
+ *    one stream stay ordered exactly as stream order promises.  Before the
+ *    wait a kernel may ask for its first data to be brought into L2.
  *  - lift_last_error() returns a detail message for the last failure of the
  *    calling thread.
  */
@@ -339,7 +340,9 @@ lift_status lift_gemv_v(int variant, int64_t M, int64_t N, float alpha, const fl
  *           distribution (0 erfcf, 1 polynomial, 2 polynomial on
  *           approximate instructions)
  *  cluster  CTAs per cluster (1 = none)
- *  passes   1: last-CTA combine in the same launch; 2: second kernel;
+ *  passes   1: last-CTA combine in the same launch (compensated sums and
+ *           the mixed-precision asum of 16 MB or more: a second kernel, the
+ *           same bits); 2: second kernel;
  *           3, 4 (gemv-T): second kernel, and the rows of a block folded
  *           in shorter groups between compensated adds (16 instead of 32; 4:
  *           pairs in blocks of 5 to 40 rows)
@@ -444,10 +447,11 @@ lift_status lift_set_policy(int policy, const char* path);
 lift_status lift_tune_stats(int64_t* tuned_shapes, int64_t* timed_launches);
 /* Force `variant` for `op` (-1 clears the override). */
 lift_status lift_set_variant(int op, int variant);
-/* (A reduction of up to 2^20 elements that is called outside stream capture
- * runs the one-launch form of this variant's tiles: the same bits.)
- * The variant the current policy would use for a dense call (aligned
- * pointers, lda = N).  M, N: gemv / gemv-T shape (else 0). */
+/* The variant the current policy would use for a dense call (aligned
+ * pointers, lda = N).  M, N: gemv / gemv-T shape (else 0).  (An asum, dot,
+ * nrm2 or sum of up to 2^20 elements that the FIXED policy picks outside
+ * stream capture runs the one-launch form of the reported variant's tiles:
+ * the same bits.) */
 lift_status lift_pick(int op, int64_t n, int64_t M, int64_t N, int* variant);
 
 /* The LIFT_NUM_FEATURES cost-model features of a call, written to

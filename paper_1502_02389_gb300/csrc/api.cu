@@ -207,8 +207,7 @@ std::vector<Variant>& registry(int op) {
 }
 
 // The grid of a kernel on a device is a fact of the hardware, so a thread may
-// keep what it has looked up (g_known); the shared map below is for the first
-// time.
+// keep what it has looked up; the shared map below is for the first time.
 static int64_t persistent_grid_shared(const void* kernel, int threads, size_t smem, int cluster);
 
 int64_t persistent_grid(const void* kernel, int threads, size_t smem, int cluster) {
@@ -385,7 +384,11 @@ static bool eligible(int op, const Variant& v, const Args& a) {
 //    2000 rows on (2400 x 32768: 49 against 53 for the split rows); below
 //    that the rows are split over CTAs (600 x 131072: 48 against 80;
 //    64 x 32768: 4.3 against 16).  A few rows of one ring's length stay with
-//    the ring: no second pass (64 x 4096: 3.0 against 3.5).
+//    the ring, which has no second pass and does not need many CTAs for so
+//    little (ring, split: 64 x 4096 2.6, 3.3; 500 x 2048 3.2, 4.4; 1000 x 2048
+//    4.1, 4.4; 1500 x 2048 4.5, 3.9; 1999 x 3072 7.1, 6.4; 300 x 6144 3.9, 4.2;
+//    500 x 6144 5.4, 4.6; 1999 x 6144 10.8, 8.3): split from 1000 rows on below
+//    4096 columns, from 500 below 8192.
 //  * N < 2048: a warp per row, as the ring's stages would be mostly empty
 //    (20000 x 1024: 16.1 against 17; 80000 x 64: 16.9 against 44);
 //    8-float loads from 256 columns on, where one row fills a warp's load, to

@@ -117,8 +117,8 @@ void register_mixed(std::vector<Variant>* ops);   // ops[LIFT_OP_*]
 int64_t persistent_grid(const void* kernel, int threads, size_t smem, int cluster);
 
 // pdl: launch as a programmatic dependent of the kernel before it on the
-// stream (the kernel must execute griddepcontrol.wait before its first
-// global memory access; see pdl_wait).
+// stream (the kernel must execute griddepcontrol.wait before it reads or
+// writes global memory; see pdl_wait.  A prefetch into L2 may come before).
 lift_status launch_config(const void* kernel, dim3 grid, dim3 block, size_t smem,
                           int cluster, cudaStream_t s, void** args, bool pdl = false);
 
@@ -147,8 +147,10 @@ __device__ __forceinline__ void prefetch_l2(const void* p, int64_t bytes) {
   if (bytes > 0 && e > a)
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a), "r"((uint32_t)(e - a)) : "memory");
 }
-// CTAs of a one-CTA-per-tile grid that prefetch: about the first wave
-constexpr unsigned kPrefetchCtas = 1216;
+// CTAs of a one-CTA-per-tile grid that prefetch: the first wave at eight CTAs
+// on each of this part's 152 SMs, the most that any of these kernels has
+// resident.  Only the first wave can be waiting while the previous call drains.
+constexpr unsigned kPrefetchCtas = 8 * 152;
 // v, as a value of its own: what is computed from it before pdl_wait is not
 // kept in registers for the kernel's body (four to twelve more registers, and
 // with them a CTA per SM, cost the compensated dot and the bf16 dot 2 %).

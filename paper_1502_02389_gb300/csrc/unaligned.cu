@@ -21,8 +21,9 @@
 // the 4-byte forms with a few loads per thread much more.
 //
 // Bound by DRAM.  Measured, us per call, dot_comp + axpy + nrm2 + asum of
-// 2^24 + 43 elements, offsets 1 and 3: 94.9 with the 4-byte forms, 80.6 here
-// (69 at the copy bandwidth); alone in a graph: axpy 38.3 -> 30.5, scal 24.9
+// 2^24 + 43 elements, offsets 1 and 3: 94.9 with the 4-byte forms, 80.6 with
+// these and 75.3 with their prefetches and second kernel (69 at the copy
+// bandwidth); alone in a graph: axpy 38.3 -> 30.5, scal 24.9
 // -> 21.3, nrm2 17.3 -> 15.3, dot 25.6 -> 23.6, dot_comp 25.3 -> 24.2.
 #include "comp_sum.cuh"
 
