@@ -50,10 +50,10 @@
  *    Calls on more than 8 streams at once share slots and can race (and
  *    after 4096 distinct stream handles the assignment starts afresh).
  *    Beside the slot each of the first 256 streams of a device has scratch
- *    of its own, which the fp32 asum, dot, nrm2 and sum and the gemv of few
- *    rows use, so these do not race however many streams there are; on later
- *    streams gemv runs forms that keep no scratch.  gemv-T, slices, and the
- *    compensated and mixed-precision reductions use the slot.
+ *    of its own, which the one-launch fp32 reductions (up to 2^20 elements,
+ *    outside stream capture) and the gemv of few rows use, so these do not
+ *    race however many streams there are; on later streams gemv runs forms
+ *    that keep no scratch.  Everything else uses the slot.
  *  - Most kernels are launched as programmatic dependents of the kernel
  *    before them on the stream: their CTAs may be scheduled while that
  *    kernel still runs, but each waits for it to complete (and for its

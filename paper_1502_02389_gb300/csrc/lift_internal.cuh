@@ -38,8 +38,8 @@ struct Workspace {
 // tickets.
 constexpr int kWsSlots = 8;
 // Small scratch of a stream's own beside its slot, for the first kOwnStreams
-// streams of a device: the partials of an fp32 reduction or of a gemv with
-// split rows, one per row and CTA at most (5472 on 152 SMs), and a ticket
+// streams of a device: the partials of a one-launch fp32 reduction or of a gemv
+// with split rows, one per row and CTA at most (5472 on 152 SMs), and a ticket
 // behind them (asum of 2^20: 3.90 us so, 4.10 with the tickets in an array of
 // their own).  A default gemv keeps no scratch that another stream writes,
 // however many streams there are.

@@ -1,5 +1,5 @@
 """More streams than workspace slots: default gemv calls of few rows, and
-small and large fp32 reductions, keep their partials in scratch of the
+fp32 reductions of one launch, keep their partials in scratch of the
 stream's own, so calls on many streams at once give the bits of the same
 calls one after another; streams beyond the last own scratch run forms that
 keep none.  In a process of its own: the streams stay assigned until the
@@ -47,7 +47,7 @@ _CHILD = textwrap.dedent(
         L.lift_gemv(6, 119999, 1.0, A, 119999, x.data_ptr() + 4, 0.0, out[6:12], s)
         L.lift_asum(z, 1 << 18, out[12:13], s)
         L.lift_dot(z, z, 3 << 18, out[13:14], s)
-        L.lift_sum(z, 1 << 21, out[14:15], s)
+        L.lift_sum(z, 1 << 20, out[14:15], s)
 
     g = torch.Generator(device="cuda").manual_seed(1)
     rnd = lambda *n: torch.randn(*n, device="cuda", generator=g)
