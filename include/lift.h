@@ -53,7 +53,9 @@
  *    of its own, which the one-launch fp32 reductions (up to 2^20 elements,
  *    outside stream capture) and the gemv of few rows use, so these do not
  *    race however many streams there are; on later streams gemv runs forms
- *    that keep no scratch.  Everything else uses the slot.
+ *    that keep no scratch.  A captured gemv has scratch of its capture's
+ *    own (for the first 768 captures, then the same).  Everything else uses
+ *    the slot.
  *  - Most kernels are launched as programmatic dependents of the kernel
  *    before them on the stream: their CTAs may be scheduled while that
  *    kernel still runs, but each waits for it to complete (and for its
@@ -121,10 +123,8 @@ typedef enum {
  * on it: 8 slots of partials and tickets (about 17 MiB each), one per
  * stream that launches work on the device (a stream takes the next slot on
  * its first call; beyond 8 streams slots are shared in turn), so calls on
- * up to 8 streams may run at the same time.  A CUDA graph keeps the slot and
- * the scratch of the stream it was captured on, also those of its gemv calls:
- * replays of graphs captured on one stream must not overlap on others.
- * Must be called (once per device) before
+ * up to 8 streams may run at the same time.  A CUDA graph keeps the slot of
+ * the stream it was captured on.  Must be called (once per device) before
  * any other call on that device, outside CUDA graph capture.  Calling it
  * again is a no-op; calls from several threads at once set the device up
  * once.

@@ -88,6 +88,22 @@ Workspace* stream_workspace(DeviceState* st, cudaStream_t stream, int* own) {
   return &slot(st, it->second.slot);
 }
 
+// Index of the own scratch of a gemv that is being captured on `stream` in
+// capture `id` (a capture may fork streams, whose calls may run side by side),
+// -1 without.
+static std::map<std::tuple<DeviceState*, unsigned long long, cudaStream_t>, int> g_capture_own;
+
+static int capture_scratch(DeviceState* st, unsigned long long id, cudaStream_t stream) {
+  std::lock_guard<std::mutex> lk(g_mu);
+  const auto key = std::make_tuple(st, id, stream);
+  auto it = g_capture_own.find(key);
+  if (it == g_capture_own.end()) {
+    if (st->captured >= kOwnCaptures) return -1;
+    it = g_capture_own.emplace(key, kOwnStreams + st->captured++).first;
+  }
+  return it->second;
+}
+
 static void free_slots(DeviceState* st) {
   for (int i = 0; i < kWsSlots; ++i) {
     Workspace& w = slot(st, i);
@@ -136,7 +152,7 @@ static lift_status init_device(int device) {
     w.capacity = kPartialCapacity;
     w.capacity64 = kPartial64Capacity;
   }
-  const size_t own_bytes = kOwnStreams * kOwnWords * sizeof(float);
+  const size_t own_bytes = (kOwnStreams + kOwnCaptures) * kOwnWords * sizeof(float);
   if (rc == LIFT_OK) rc = cuda_check(cudaMalloc(&st->own, own_bytes), "workspace");
   if (rc == LIFT_OK) rc = cuda_check(cudaMemset(st->own, 0, own_bytes), "memset");
   if (rc == LIFT_OK) rc = cuda_check(cudaDeviceSynchronize(), "init sync");
@@ -879,17 +895,32 @@ static lift_status run(int op, int variant, const Args& a0, void* stream) {
   Args a = a0;
   int own = -1;
   a.ws = stream_workspace(st, s, &own);
-  a.must_share = own < 0;
-  if (own >= 0) {
-    a.own = st->own + own * kOwnWords;
-    a.own_ticket = reinterpret_cast<unsigned*>(a.own + kOwnFloats);
-  }
+  auto use = [&](int index) {
+    a.must_share = index < 0;
+    a.own = index < 0 ? nullptr : st->own + index * kOwnWords;
+    a.own_ticket = index < 0 ? nullptr : reinterpret_cast<unsigned*>(a.own + kOwnFloats);
+  };
+  use(own);
+  // a captured gemv that may split rows takes its capture's scratch instead
+  auto capture = [&] {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    unsigned long long id = 0;
+    if (cudaStreamGetCaptureInfo(s, &cs, &id) != cudaSuccess) cudaGetLastError();
+    if (cs != cudaStreamCaptureStatusActive) return false;
+    use(capture_scratch(st, id, s));
+    return true;
+  };
+  const bool looked = op == LIFT_OP_GEMV && own < 0;
+  if (looked) capture();
   // A call of two launches leaves partials in the slot between them, and a
   // timing of candidates uses the slot on a stream of its own: another host
   // thread's call on this stream comes before or after all of it.
   std::lock_guard<std::mutex> slot_lk(*a.ws->mu);
   const Variant* v = nullptr;
   lift_status rc = resolve(op, variant, a, &v, s, true);
+  if (rc == LIFT_OK && op == LIFT_OP_GEMV && !looked && v->info.passes == 2 && capture() &&
+      a.must_share)
+    rc = resolve(op, variant, a, &v, s, true);
   if (rc != LIFT_OK) return rc;
   return v->launch(*v, a, s);
 }
@@ -987,6 +1018,7 @@ lift_status lift_finalize(void) {
   g_states.clear();
   g_slot_of.clear();
   g_next_slot.clear();
+  g_capture_own.clear();
   if (prev >= 0) cudaSetDevice(prev);
   return LIFT_OK;
 }
@@ -1025,7 +1057,8 @@ int lift_read_status(int clear) {
     bool ok = cudaDeviceSynchronize() == cudaSuccess;
     for (int i = 0; i < kWsSlots && ok; ++i)
       ok = cudaMemset(slot(st, i).tickets, 0, kTicketSlots * sizeof(unsigned)) == cudaSuccess;
-    ok = ok && cudaMemset(st->own, 0, kOwnStreams * kOwnWords * sizeof(float)) == cudaSuccess;
+    ok = ok && cudaMemset(st->own, 0, (kOwnStreams + kOwnCaptures) * kOwnWords * sizeof(float)) ==
+                   cudaSuccess;
     ok = ok && cudaMemset(st->ws.status, 0, sizeof(int)) == cudaSuccess &&
          cudaDeviceSynchronize() == cudaSuccess;
     if (!ok) return LIFT_ERR_CUDA;

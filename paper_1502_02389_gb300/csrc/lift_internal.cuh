@@ -42,8 +42,9 @@ constexpr int kWsSlots = 8;
 // with split rows, one per row and CTA at most (5472 on 152 SMs), and a ticket
 // behind them (asum of 2^20: 3.90 us so, 4.10 with the tickets in an array of
 // their own).  A default gemv keeps no scratch that another stream writes,
-// however many streams there are.
-constexpr int kOwnStreams = 256;
+// however many streams there are, nor, for the first kOwnCaptures captures, that
+// another graph does: graphs captured on one stream may be replayed on several.
+constexpr int kOwnStreams = 256, kOwnCaptures = 768;
 constexpr int64_t kOwnWords = 8192, kOwnFloats = kOwnWords - 32;
 
 struct DeviceState {
@@ -52,8 +53,8 @@ struct DeviceState {
   Workspace ws;                    // slot 0 (also the capacities and the status word)
   Workspace more[kWsSlots - 1];    // slots 1 ..
   std::mutex slot_mu[kWsSlots];    // the slots' mutexes
-  float* own = nullptr;            // kOwnStreams * kOwnWords (the tickets are 0 between calls)
-  int owned = 0;                   // streams that have scratch of their own
+  float* own = nullptr;            // (kOwnStreams + kOwnCaptures) * kOwnWords; tickets are 0 between calls
+  int owned = 0, captured = 0;     // streams and captures that have scratch of their own
 };
 
 DeviceState* current_state();  // state of the current device, or nullptr

@@ -2,7 +2,8 @@
 fp32 reductions of one launch, keep their partials in scratch of the
 stream's own, so calls on many streams at once give the bits of the same
 calls one after another; streams beyond the last own scratch run forms that
-keep none.  In a process of its own: the streams stay assigned until the
+keep none, and graphs captured on one stream may be replayed side by side.
+In a process of its own: the streams stay assigned until the
 library is finalised."""
 import os
 import subprocess
@@ -73,6 +74,24 @@ _CHILD = textwrap.dedent(
         assert torch.equal(got, want[None].expand_as(got)), first
         ref = torch.stack([(A.double() @ x[:120000].double()) for A, x, _ in data])
         assert torch.all((want[:, :6] - ref).abs() <= 1e-5 * ref.abs().max())
+    # graphs captured on one stream, replayed side by side on others
+    cap, side = torch.cuda.Stream(), [torch.cuda.Stream() for _ in range(3)]
+    out = torch.zeros(3, 40, 12, device="cuda")
+    graphs = []
+    for k in range(3):
+        A, x, _ = data[k]
+        gr = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(gr, stream=cap):
+            for i in range(40):
+                L.lift_gemv(6, 120000, 1.0, A, 120000, x, 0.0, out[k, i][0:6], cap)
+                L.lift_gemv(6, 119999, 1.0, A, 119999, x.data_ptr() + 4, 0.0, out[k, i][6:12], cap)
+        graphs.append(gr)
+    for _ in range(20):
+        for gr, s in zip(graphs, side):
+            with torch.cuda.stream(s):
+                gr.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out, want[:3, None, :12].expand_as(out))
     assert L.lift_read_status() == 0
     print("OK")
     """
