@@ -120,10 +120,10 @@ typedef enum {
  * ------------------------------------------------------------------------ */
 
 /* Set up `device`: query its SM count and allocate the reduction workspace
- * on it: 8 slots of partials and tickets (about 17 MiB each), one per
- * stream that launches work on the device (a stream takes the next slot on
- * its first call; beyond 8 streams slots are shared in turn), so calls on
- * up to 8 streams may run at the same time.  A CUDA graph keeps the slot of
+ * on it: 8 slots of partials and tickets (about 17 MiB each), and 32 MiB of
+ * scratch for single streams and captures.  A stream that launches work on
+ * the device takes the next slot on its first call (beyond 8 streams slots
+ * are shared in turn), so calls on up to 8 streams may run at the same time.  A CUDA graph keeps the slot of
  * the stream it was captured on.  Must be called (once per device) before
  * any other call on that device, outside CUDA graph capture.  Calling it
  * again is a no-op; calls from several threads at once set the device up
